@@ -49,12 +49,13 @@ typedef enum {
 
 /* Arithmetic of the FFTs and pointwise steps.  The integrator state and its step control
  * are FP64 in every mode.
- *   SCFFT_PREC_F64   FP64 transforms; FP64 stage sums.
+ *   SCFFT_PREC_F64   FP64 spectra and fields, FP64 stage sums.  The transforms run on 64-bit
+ *                    integers with an exponent per block of values (nearer to exact arithmetic
+ *                    than FP64 transforms), or, with every axis at most 32, in FP64.  Values below
+ *                    2.2e-308 count as zero; an infinity or a NaN makes the pencils it meets NaN.
  *   SCFFT_PREC_F32   FP32 transforms and stages, FP64 state with compensated sums.
- *   SCFFT_PREC_DF64  double-float transforms (each value an unevaluated sum of two FP32
- *                    numbers, a 48-bit significand, FP32's exponent range: FP64-equivalent
- *                    accuracy on the FP32 pipes); the node-wise law in FP64; FP64 stage sums.
- *                    Its buffers, entry points and results are those of SCFFT_PREC_F64. */
+ *   SCFFT_PREC_DF64  the same as SCFFT_PREC_F64 (kept for programs that ask for it: a faster
+ *                    FP64-equivalent form, which the FP64 passes have become). */
 #define SCFFT_PREC_F64 0
 #define SCFFT_PREC_F32 1
 #define SCFFT_PREC_DF64 2

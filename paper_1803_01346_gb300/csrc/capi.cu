@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "scfft.h"
+#include "fx64.cuh"
 #include "scfft_internal.cuh"
 
 using namespace scfft;
@@ -36,7 +37,6 @@ struct scfft_ctx {
   cudaStream_t st = nullptr;
   Work<float> wf;
   Work<double> wd;
-  Work<dfloat> wq;  // double-float FFT passes (SCFFT_PREC_DF64)
   int box[4] = {0, 0, 0, 0};  // bounding box of Omega's nodes: y in [box0, box1) (even), z in [box2, box3)
   Ctrl* ctrl = nullptr;        // device
   PointParams* ppd = nullptr;  // device copy of the current rhs's PointParams
@@ -151,13 +151,11 @@ bool grid_ok(int n) { return n == 16 || n == 32 || n == 48 || n == 64 || n == 96
 template <typename T> Work<T>& work(scfft_ctx* c);
 template <> Work<float>& work<float>(scfft_ctx* c) { return c->wf; }
 template <> Work<double>& work<double>(scfft_ctx* c) { return c->wd; }
-template <> Work<dfloat>& work<dfloat>(scfft_ctx* c) { return c->wq; }
 
-// Calls f with a value of the context's FFT element type: float (SCFFT_PREC_F32), double
-// (SCFFT_PREC_F64) or dfloat (SCFFT_PREC_DF64).
+// Calls f with a value of the context's FFT element type: float (SCFFT_PREC_F32) or double
+// (SCFFT_PREC_F64, SCFFT_PREC_DF64).
 template <typename F> auto by_prec(const scfft_ctx* c, F&& f) {
   if (c->opt.precision == SCFFT_PREC_F32) return f(float{});
-  if (c->opt.precision == SCFFT_PREC_DF64) return f(dfloat{});
   return f(double{});
 }
 
@@ -267,6 +265,7 @@ template <typename T> scfft_status alloc_work(scfft_ctx* c) {
   CK(cudaMalloc(&w.Hd[1], sizeof(T) * 3 * N));
   CK(cudaMalloc(&w.kap, sizeof(T) * 3 * (size_t)(g.nx + 1) * (g.ny + 1) * (g.nz + 1)));
   if constexpr (sizeof(T) == 4) CK(cudaMalloc(&w.kap4, sizeof(float4) * (size_t)(g.nx + 1) * (g.ny + 1) * (g.nz + 1)));
+  if (std::is_same<T, double>::value && fixed_point_grid(g)) CK(cudaMalloc(&w.ek, sizeof(int) * (size_t)(g.nx + 1) * (g.ny + 1)));
   const int n[3] = {g.nx, g.ny, g.nz};
   const double sig = c->opt.sigma_scale * 0.5 *
                      sqrt(pow(2 * c->L[0] / g.nx, 2) + pow(2 * c->L[1] / g.ny, 2) + pow(2 * c->L[2] / g.nz, 2));
@@ -284,8 +283,36 @@ template <typename T> scfft_status alloc_work(scfft_ctx* c) {
     CK(cudaMalloc(&w.st[a], sizeof(T) * len));
     CK(cudaMemcpy(w.kt[a], kt.data(), sizeof(T) * len, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(w.st[a], st.data(), sizeof(T) * len, cudaMemcpyHostToDevice));
+    if constexpr (std::is_same<T, double>::value) {
+      if (a == 2 && fixed_point_grid(g)) {  // S and S k along z as integers |t| < 2^62 (fx64.cuh)
+        for (int q = 0; q < 2; ++q) {
+          std::vector<long long> t(len);
+          double m = 0.0;
+          for (int i = 0; i < len; ++i) m = std::max(m, fabs(q ? st[i] * kt[i] : st[i]));
+          frexp(m, &w.ze[q]);
+          for (int i = 0; i < len; ++i) t[i] = llrint(ldexp(q ? st[i] * kt[i] : st[i], 62 - w.ze[q]));
+          CK(cudaMalloc(&w.zt[q], sizeof(long long) * len));
+          CK(cudaMemcpy(w.zt[q], t.data(), sizeof(long long) * len, cudaMemcpyHostToDevice));
+        }
+      }
+    }
     for (int pad = 0; pad < 2; ++pad) {
       const int Lt = pad ? 2 * n[a] : n[a];
+      if constexpr (std::is_same<T, double>::value) {
+        if (fixed_point_grid(g)) {
+          // the fixed-point passes' twiddles: 2^62 (cos, sin), as halves whose low one is odd
+          std::vector<int4> fw(Lt);
+          for (int m = 0; m < Lt; ++m) {
+            const long double ang = 2.0L * 3.14159265358979323846264338327950288L * m / Lt;
+            const long long cs = llrintl(ldexpl(cosl(ang), 62)) | 1, sn = llrintl(ldexpl(sinl(ang), 62)) | 1;
+            fw[m] = make_int4(fx_hi(cs), fx_lo(cs), fx_hi(sn), fx_lo(sn));
+          }
+          int4** fd = pad ? &w.fxp[a] : &w.fxu[a];
+          CK(cudaMalloc(fd, sizeof(int4) * Lt));
+          CK(cudaMemcpy(*fd, fw.data(), sizeof(int4) * Lt, cudaMemcpyHostToDevice));
+          continue;
+        }
+      }
       std::vector<V> tw(Lt);
       for (int m = 0; m < Lt; ++m) {
         const long double ang = 2.0L * 3.14159265358979323846264338327950288L * m / Lt;
@@ -311,6 +338,8 @@ template <typename T> void free_work(Work<T>& w) {
   delete w.ym;
   cudaFree(w.Jd);
   for (int a = 0; a < 3; ++a) { cudaFree(w.kt[a]); cudaFree(w.st[a]); cudaFree(w.twu[a]); cudaFree(w.twp[a]); }
+  for (int a = 0; a < 3; ++a) { cudaFree(w.fxu[a]); cudaFree(w.fxp[a]); }
+  cudaFree(w.zt[0]); cudaFree(w.zt[1]); cudaFree(w.ek);
   w = Work<T>();
 }
 
@@ -1755,7 +1784,6 @@ void scfft_destroy(scfft_ctx* c) {
   if (c->hsdev) cudaFreeHost(c->hsdev);
   free_work(c->wf);
   free_work(c->wd);
-  free_work(c->wq);
   if (c->loop_exec) cudaGraphExecDestroy(c->loop_exec);
   if (c->loop_graph) cudaGraphDestroy(c->loop_graph);
   cudaFree(c->ctrl); cudaFree(c->ppd); cudaFree(c->partials); cudaFree(c->mask); cudaFree(c->ib); cudaFree(c->errbits);

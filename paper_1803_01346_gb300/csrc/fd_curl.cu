@@ -58,13 +58,13 @@ __global__ void fd_efield_kernel(Src h, const uint8_t* __restrict__ mask, const 
     const int x = (int)(i % g.nx);
     const long long r = i / g.nx;
     const int y = (int)(r % g.ny), z = (int)(r / g.ny);
-    typedef typename acc_of<T>::type A;  // the law's arithmetic (FP64 for double-float)
+    typedef T A;
     T jt[3];
     curl_at<T>([&](long long k) { return h.at(k); }, x, y, z, g, inv2d0, inv2d1, inv2d2, jt);
-    const A j[3] = {to_acc(jt[0]), to_acc(jt[1]), to_acc(jt[2])};
+    const A j[3] = {jt[0], jt[1], jt[2]};
     A f[3];
     if (mask[i]) {
-      A jcv = jcmap ? to_acc(jcmap[i]) : (A)pp.jc;
+      A jcv = jcmap ? jcmap[i] : (A)pp.jc;
       A a[3] = {(A)1, (A)1, (A)1};
       if (pp.law) {
         if (pp.kim_h0 > 0) {
@@ -79,9 +79,9 @@ __global__ void fd_efield_kernel(Src h, const uint8_t* __restrict__ mask, const 
     } else {
       f[0] = f[1] = f[2] = (A)pp.rho_out;
     }
-    out[i] = from_acc<T>(f[0] * j[0]);
-    out[N + i] = from_acc<T>(f[1] * j[1]);
-    out[2 * N + i] = from_acc<T>(f[2] * j[2]);
+    out[i] = f[0] * j[0];
+    out[N + i] = f[1] * j[1];
+    out[2 * N + i] = f[2] * j[2];
   }
 }
 
@@ -189,7 +189,6 @@ cudaError_t launch_fd_curl_mask(const Launch<T>& L, T* out, const double* d, boo
   template cudaError_t launch_fd_curl_mask<T>(const Launch<T>&, T*, const double*, bool);
 INST_FD(float)
 INST_FD(double)
-INST_FD(dfloat)
 #undef INST_FD
 
 }  // namespace scfft

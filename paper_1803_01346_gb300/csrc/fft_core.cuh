@@ -1,19 +1,11 @@
-// fft_core.cuh - shared-memory mixed-radix FFT building blocks for sm_103a.
+// fft_core.cuh - complex arithmetic and the small DFTs of the FFT passes for sm_103a.
 //
-// A CTA holds a batch of pencils in shared memory and transforms them with a
-// Stockham auto-sort sequence of radix-R stages (R in {2,3,4,8,12,16}); each
-// stage keeps its R points in registers (small DFT below), applies the
-// inter-stage twiddles from a per-length table staged in shared memory, and
-// writes the other buffer of a ping-pong pair, so the result comes out in
-// natural order without a bit-reversal pass.  Shared-memory layout of a batch:
-//   element e of pencil p lives at (p / PT) * CS + e * ES + (p % PT)
-// (PT pencils per "component" side by side, odd ES so that threads walking
-// consecutive pencils hit distinct banks).
+// Every pass transforms its pencils in one or two register stages of R points (R in {2,3,4,8,12,16},
+// the DFTs below) with a shared-memory transpose between them.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "df64.cuh"
 
 namespace scfft {
 
@@ -21,7 +13,15 @@ namespace scfft {
 template <typename T> struct cplx_of;
 template <> struct cplx_of<float> { typedef float2 type; };
 template <> struct cplx_of<double> { typedef double2 type; };
-template <> struct cplx_of<dfloat> { typedef dfloat2 type; };
+
+// complex 64-bit fixed point (fx64.cuh)
+struct __align__(16) fxc {
+  long long x, y;
+};
+#define FXHD __host__ __device__ __forceinline__
+FXHD fxc mk(long long a, long long b) { fxc r; r.x = a; r.y = b; return r; }
+FXHD fxc operator+(fxc a, fxc b) { return mk(a.x + b.x, a.y + b.y); }
+FXHD fxc operator-(fxc a, fxc b) { return mk(a.x - b.x, a.y - b.y); }
 
 __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
@@ -84,25 +84,6 @@ template <typename V, int R, bool INV> struct TwiddleConst {
       return INV ? mk(h * (sc * a.x - ss * a.y), h * (ss * a.x + sc * a.y))
                  : mk(h * (sc * a.x + ss * a.y), h * (sc * a.y - ss * a.x));
     }
-    return INV ? mk(a.x * c - a.y * s, a.x * s + a.y * c) : mk(a.x * c + a.y * s, a.y * c - a.x * s);
-  }
-};
-// double-float: the constants are the nearest double-floats of the FP64 values (folded at
-// compile time); the sign flips of the odd multiples of pi/4 are negations, not products
-template <int R, bool INV> struct TwiddleConst<dfloat2, R, INV> {
-  static __device__ __forceinline__ dfloat2 apply(dfloat2 a, int m) {
-    const int q = ((2 * m * 24 / R) % 48 + 48) % 48;
-    if (q == 0) return a;
-    if (q == 24) return mk(-a.x, -a.y);
-    if (q == 12) return INV ? mk(-a.y, a.x) : mk(a.y, -a.x);
-    if (q == 36) return INV ? mk(a.y, -a.x) : mk(-a.y, a.x);
-    if (q % 12 == 6) {
-      const dfloat h(0.7071067811865475244008444);
-      const dfloat ax = cos24(q) > 0 ? a.x : -a.x, ay = cos24(q) > 0 ? a.y : -a.y;  // sign(c) a
-      const dfloat bx = sin24(q) > 0 ? a.x : -a.x, by = sin24(q) > 0 ? a.y : -a.y;  // sign(s) a
-      return INV ? mk(h * (ax - by), h * (bx + ay)) : mk(h * (ax + by), h * (ay - bx));
-    }
-    const dfloat c(cos24(q)), s(sin24(q));
     return INV ? mk(a.x * c - a.y * s, a.x * s + a.y * c) : mk(a.x * c + a.y * s, a.y * c - a.x * s);
   }
 };
@@ -265,81 +246,6 @@ template <bool INV, typename V> struct DFTh<16, INV, V> {
 template <int R, bool INV, bool HALF, typename V> __device__ __forceinline__ void dft_maybe_half(V* v) {
   if constexpr (HALF) DFTh<R, INV, V>::run(v);
   else DFT<R, INV, V>::run(v);
-}
-
-// ---------------------------------------------------------------- plans
-struct FftPlan {
-  int L;       // transform length
-  int ns;      // number of stages
-  int r[4];    // radix of each stage (product = L)
-};
-
-// Batch geometry in shared memory (see the header comment).
-struct Batch {
-  int P;   // pencils
-  int PT;  // pencils per component block
-  int ES;  // element stride (in complex elements)
-  int CS;  // component block stride
-};
-
-__device__ __forceinline__ int pbase(const Batch& b, int p) { return (p / b.PT) * b.CS + (p % b.PT); }
-
-// One Stockham stage: for j in [0, L/R), k = j mod Ns,
-//   v_q = src[j + q L/R] * W_{Ns R}^{q k};  v = DFT_R(v);  dst[(j/Ns) Ns R + k + q Ns] = v_q
-template <int R, bool INV, typename V>
-__device__ __forceinline__ void stockham_stage(const V* __restrict__ src, V* __restrict__ dst, const V* __restrict__ tw,
-                                               int L, int Ns, const Batch& b) {
-  const int LR = L / R;
-  const int tasks = b.P * LR;
-  const int twstep = L / (Ns * R);  // W_{Ns R}^{qk} = W_L^{q k twstep}
-  for (int t = threadIdx.x; t < tasks; t += blockDim.x) {
-    const int p = t % b.P;
-    const int j = t / b.P;
-    const int k = j % Ns;
-    const int base = pbase(b, p);
-    V v[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = src[base + (j + q * LR) * b.ES];
-    if (Ns > 1) {
-#pragma unroll
-      for (int q = 1; q < R; ++q) {
-        const V w = tw[q * k * twstep];
-        v[q] = INV ? cmulc(v[q], w) : cmul(v[q], w);
-      }
-    }
-    DFT<R, INV, V>::run(v);
-    const int d0 = (j / Ns) * Ns * R + k;
-#pragma unroll
-    for (int q = 0; q < R; ++q) dst[base + (d0 + q * Ns) * b.ES] = v[q];
-  }
-}
-
-// Full transform of every pencil of the batch.  Data starts in buf[0]; returns
-// the index (0/1) of the buffer holding the result.  Ends with __syncthreads().
-template <bool INV, typename V>
-__device__ int fft_batch(V* buf0, V* buf1, const V* tw, const FftPlan& pl, const Batch& b) {
-  V* src = buf0;
-  V* dst = buf1;
-  int Ns = 1;
-  int which = 0;
-  for (int s = 0; s < pl.ns; ++s) {
-    const int R = pl.r[s];
-    switch (R) {
-      case 2: stockham_stage<2, INV>(src, dst, tw, pl.L, Ns, b); break;
-      case 3: stockham_stage<3, INV>(src, dst, tw, pl.L, Ns, b); break;
-      case 4: stockham_stage<4, INV>(src, dst, tw, pl.L, Ns, b); break;
-      case 8: stockham_stage<8, INV>(src, dst, tw, pl.L, Ns, b); break;
-      case 12: stockham_stage<12, INV>(src, dst, tw, pl.L, Ns, b); break;
-      default: stockham_stage<16, INV>(src, dst, tw, pl.L, Ns, b); break;
-    }
-    __syncthreads();
-    V* t = src;
-    src = dst;
-    dst = t;
-    which ^= 1;
-    Ns *= R;
-  }
-  return which;
 }
 
 }  // namespace scfft

@@ -20,6 +20,7 @@
 
 #include <mutex>
 
+#include "fx64.cuh"
 #include "scfft.h"
 #include "scfft_internal.cuh"
 
@@ -53,9 +54,10 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Per-grid tables, written on the device: twiddles W_L^m for L = nx, ny, nz;
 // derivative wavenumbers pi m / L_a (0 on the Nyquist entry) and smoothing
-// factors exp(-sigma^2 k^2 / 2) for the x half spectrum and the full y, z axes.
-__global__ void noalloc_tables(double2* tw, double* kt, double* st, int nx, int ny, int nz, double Lx, double Ly,
-                               double Lz, double sigma) {
+// factors exp(-sigma^2 k^2 / 2) for the x half spectrum and the full y, z axes.  fw, zt: the same
+// twiddles, and S and S k along z, as integers for the fixed-point passes (Work::fxu, Work::zt).
+__global__ void noalloc_tables(double2* tw, double* kt, double* st, int4* fw, long long* zt, int e1, int e2, int nx,
+                               int ny, int nz, double Lx, double Ly, double Lz, double sigma) {
   const int n[3] = {nx, ny, nz};
   const double L[3] = {Lx, Ly, Lz};
   int toff = 0, koff = 0;
@@ -64,6 +66,8 @@ __global__ void noalloc_tables(double2* tw, double* kt, double* st, int nx, int 
       double s, c;
       sincospi(2.0 * m / n[a], &s, &c);
       tw[toff + m] = make_double2(c, -s);
+      const long long ci = __double2ll_rn(ldexp(c, 62)) | 1, si = __double2ll_rn(ldexp(s, 62)) | 1;
+      fw[toff + m] = make_int4(fx_hi(ci), fx_lo(ci), fx_hi(si), fx_lo(si));
     }
     const int len = a == 0 ? n[0] / 2 + 1 : n[a];
     for (int i = threadIdx.x; i < len; i += blockDim.x) {
@@ -71,6 +75,10 @@ __global__ void noalloc_tables(double2* tw, double* kt, double* st, int nx, int 
       const double k = M_PI * m / L[a];
       kt[koff + i] = (i == n[a] / 2) ? 0.0 : k;
       st[koff + i] = exp(-0.5 * sigma * sigma * k * k);
+      if (a == 2) {
+        zt[i] = __double2ll_rn(ldexp(st[koff + i], 62 - e1));
+        zt[nz + i] = __double2ll_rn(ldexp(st[koff + i] * kt[koff + i], 62 - e2));
+      }
     }
     toff += n[a];
     koff += len;
@@ -91,12 +99,14 @@ extern "C" scfft_status scfft_curl_noalloc(const scfft_grid* grid, double sigma_
   g.sxu = (grid->nx / 2 + 1 + 7) / 8 * 8;
   g.sxp = (grid->nx + 1 + 7) / 8 * 8;
   g.N = (long long)g.nx * g.ny * g.nz;
-  // carve the scratch: twiddles | wavenumbers | smoothing | half spectrum
+  // carve the scratch: twiddles | wavenumbers | smoothing | integer tables | half spectrum
   const size_t ntw = (size_t)g.nx + g.ny + g.nz;
   const size_t nk = (size_t)g.nx / 2 + 1 + g.ny + g.nz;
   const size_t off_kt = align256(ntw * sizeof(double2));
   const size_t off_st = off_kt + align256(nk * sizeof(double));
-  const size_t off_u = off_st + align256(nk * sizeof(double));
+  const size_t off_fw = off_st + align256(nk * sizeof(double));
+  const size_t off_zt = off_fw + align256(ntw * sizeof(int4));
+  const size_t off_u = off_zt + align256(2 * (size_t)g.nz * sizeof(long long));
   const size_t need = off_u + sizeof(double2) * 3 * (size_t)g.nz * g.ny * g.sxu;
   if (need > kNoAllocBytes) return SCFFT_ESIZE;
 
@@ -133,6 +143,19 @@ extern "C" scfft_status scfft_curl_noalloc(const scfft_grid* grid, double sigma_
   const double dx = 2 * grid->Lx / g.nx, dy = 2 * grid->Ly / g.ny, dz = 2 * grid->Lz / g.nz;
   const double sigma = sigma_scale * 0.5 * sqrt(dx * dx + dy * dy + dz * dz);
 
+  int4* fw = reinterpret_cast<int4*>(base + off_fw);
+  long long* zt = reinterpret_cast<long long*>(base + off_zt);
+  w.fxu[0] = fw; w.fxu[1] = fw + g.nx; w.fxu[2] = fw + g.nx + g.ny;
+  w.zt[0] = zt; w.zt[1] = zt + g.nz;
+  // exponents of the largest S and S k along z (a hair of room for the device's exp)
+  double smax = 1.0, skmax = 0.0;
+  for (int m = 0; m < g.nz / 2; ++m) {
+    const double k = M_PI * m / grid->Lz;
+    skmax = fmax(skmax, k * exp(-0.5 * sigma * sigma * k * k));
+  }
+  frexp(smax * (1 + 1e-12), &w.ze[0]);
+  frexp(skmax * (1 + 1e-12), &w.ze[1]);
+
   Launch<double> L;
   L.g = g;
   L.w = &w;
@@ -141,7 +164,7 @@ extern "C" scfft_status scfft_curl_noalloc(const scfft_grid* grid, double sigma_
   L.partials = nullptr;
   L.st = s;
   PointParams pp{};
-  noalloc_tables<<<1, 256, 0, s>>>(tw, kt, st, g.nx, g.ny, g.nz, grid->Lx, grid->Ly, grid->Lz, sigma);
+  noalloc_tables<<<1, 256, 0, s>>>(tw, kt, st, fw, zt, w.ze[0], w.ze[1], g.nx, g.ny, g.nz, grid->Lx, grid->Ly, grid->Lz, sigma);
   NCK(cudaGetLastError());
   NCK(launch_x<double>(L, X_FWD_F64, pp, f, nullptr, nullptr, 0, 0, false));
   NCK(launch_y<double>(L, false, false, false));

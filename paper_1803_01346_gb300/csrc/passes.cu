@@ -1,6 +1,6 @@
 // passes.cu - the FFT pass kernels of the right-hand side (§2, Eqs. 1-7): launch diagnostics,
 // plans, the small kernels and the kernel spectrum here; the shared-memory pass templates in
-// passes_impl.cuh, instantiated here for float and double (passes_df64.cu: dfloat).
+// passes_wide.cuh (its FP32 reverse-mode x passes are instantiated here).
 //
 // Every 3D transform is split into three batched 1D passes along x, y and z on
 // the layouts [comp][z][y][x] (real) and [comp][z][y][kx] (half spectrum,
@@ -14,7 +14,7 @@
 //               on the zero-padded grid.
 // Two real rows of one component travel as the real and imaginary parts of one
 // complex pencil in the x passes (two real transforms for one complex one).
-#include "passes_impl.cuh"
+#include "passes_wide.cuh"
 
 namespace scfft {
 
@@ -30,32 +30,6 @@ cudaError_t checked_launch(const char* what, dim3 grid, int block, size_t smem) 
 }
 
 const char* last_launch_failure() { return g_launch_fail; }
-
-// ---------------------------------------------------------------- plans
-bool length_supported(int L) {
-  switch (L) {
-    case 16: case 32: case 48: case 64: case 96: case 128: case 192: case 256: return true;
-    default: return false;
-  }
-}
-
-FftPlan make_plan(int L) {
-  FftPlan p{};
-  p.L = L;
-  auto set = [&](int a, int b) { p.ns = b ? 2 : 1; p.r[0] = a; p.r[1] = b; };
-  switch (L) {
-    case 16: set(16, 0); break;
-    case 32: set(8, 4); break;
-    case 48: set(16, 3); break;
-    case 64: set(8, 8); break;
-    case 96: set(8, 12); break;
-    case 128: set(16, 8); break;
-    case 192: set(16, 12); break;
-    case 256: set(16, 16); break;
-    default: p.ns = 0; break;
-  }
-  return p;
-}
 
 // ---------------------------------------------------------------- small kernels
 template <typename T>
@@ -135,9 +109,23 @@ __global__ void scale_convert_kernel(const double* __restrict__ src, double s, d
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     dst[i] = src[i] * s;
 }
-__global__ void scale_convert_kernel(const double* __restrict__ src, double s, dfloat* dst, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    dst[i] = dfloat(src[i] * s);
+// FP64: a column (ky, kx) of the kernel spectrum, in place, as integers K 2^(62 - ek) with
+// |K| < 2^ek over the column and its components
+__global__ void fix_columns_kernel(double* __restrict__ K, int* __restrict__ ek, long long plane, int nzp) {
+  const long long oct = plane * nzp;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < plane; i += (long long)gridDim.x * blockDim.x) {
+    double m = 0.0;
+    for (int c = 0; c < 3; ++c)
+      for (int z = 0; z < nzp; ++z) m = fmax(m, fabs(K[c * oct + z * plane + i]));
+    int e = -900;  // (a column of zeros)
+    if (m > 0.0) frexp(m, &e);
+    ek[i] = e;
+    for (int c = 0; c < 3; ++c)
+      for (int z = 0; z < nzp; ++z) {
+        double* p = K + c * oct + z * plane + i;
+        *p = __longlong_as_double(__double2ll_rn(scalbn(*p, 62 - e)) | 1);
+      }
+  }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -182,6 +170,11 @@ cudaError_t launch_kernel_spectrum(const Launch<T>& L, double Lx, double Ly, dou
   }
   scale_convert_kernel<<<grid_for(3 * oct), kThreads, 0, L.st>>>(B, 1.0 / (8.0 * (double)N), L.w->kap, 3 * oct);
   if constexpr (sizeof(T) == 4) interleave_kernel<<<grid_for(oct), kThreads, 0, L.st>>>(L.w->kap, L.w->kap4, oct);
+  if (std::is_same<T, double>::value && fixed_point_grid(g)) {
+    const long long plane = (long long)(nx + 1) * (ny + 1);
+    double* B2 = reinterpret_cast<double*>(L.w->kap);
+    fix_columns_kernel<<<grid_for(plane), kThreads, 0, L.st>>>(B2, L.w->ek, plane, nz + 1);
+  }
   return cudaGetLastError();
 }
 
@@ -191,9 +184,8 @@ cudaError_t launch_kernel_spectrum(const Launch<T>& L, double Lx, double Ly, dou
   template cudaError_t launch_kernel_spectrum<T>(const Launch<T>&, double, double, double, double, double*);
 INST(float)
 INST(double)
-INST(dfloat)
 #undef INST
-INST_PASSES(float)
-INST_PASSES(double)
+INST_PASSES_X(float)
+INST_PASSES_YZ(float)
 
 }  // namespace scfft

@@ -53,6 +53,13 @@ struct Geo {
   long long N;    // nx*ny*nz
 };
 
+// FP64: whether the grid's passes run in 64-bit fixed point (passes_fx.cuh) or, with every axis at
+// most 32, in native FP64 (passes_small.cuh): there both are bound by latency and about as fast
+// (one 16^3 curl 55 us native, 48 us fixed; the 64 x 64 x 96 right-hand side 9.6 ms native with the
+// same structure, 3.3 ms fixed), and the native passes keep the rounding that the small grids'
+// step sequences were recorded with.
+inline bool fixed_point_grid(const Geo& g) { return g.nx > 32 || g.ny > 32 || g.nz > 32; }
+
 // TMA descriptors of the FP32 padded y passes: the padded half spectrum Pd as read by the
 // forward pass (its first ny rows) and by the inverse pass (all 2ny rows).
 struct YMaps {
@@ -87,6 +94,14 @@ struct Work {
   V* twu[3] = {nullptr, nullptr, nullptr}; // twiddles W_L^m, L = nx, ny, nz
   V* twp[3] = {nullptr, nullptr, nullptr}; // twiddles, L = 2nx, 2ny, 2nz
   YMaps* ym = nullptr;   // FP32 only: TMA descriptors of the y passes (nullptr: plain-load y passes)
+  // FP64 only (fixed-point passes, fx64.cuh; kap as integers only on grids that take them): twiddles 2^62 (cos, sin) as 32-bit halves for L = n
+  // and L = 2n per axis; S and S k along z as integers with their exponents; exponent of a kernel
+  // spectrum's column (ky, kx), whose values kap holds as integers K 2^(62 - ek)
+  int4* fxu[3] = {nullptr, nullptr, nullptr};
+  int4* fxp[3] = {nullptr, nullptr, nullptr};
+  long long* zt[2] = {nullptr, nullptr};
+  int ze[2] = {0, 0};
+  int* ek = nullptr;
   T* Jd = nullptr;       // [3][N] masked stencil curl of the iterate (local-stencil curl option only)
   Sched sched;           // FP32 only: launch schedule of the register passes
 };
@@ -150,11 +165,11 @@ struct Launch {
   bool use_box = false;
 };
 
-// Pass launchers (defined in passes.cu, instantiated for float, double and dfloat).
+// Pass launchers (instantiated for float and double).
 template <typename T> cudaError_t launch_x(const Launch<T>& L, XMode mode, const PointParams& pp,
                                            const double* src_f64, double* dst_f64, const double* warm,
                                            int in_buf, int out_buf, bool check_done);
-// X_PAD_F64 with its real input rows in the pass's own type (FP64 and double-float passes)
+// X_PAD_F64 with its real input rows in the pass's own type (FP64 passes)
 template <typename T> cudaError_t launch_x_pad_rows(const Launch<T>& L, const PointParams& pp, const T* rows,
                                                     bool check_done);
 template <typename T> cudaError_t launch_y(const Launch<T>& L, bool padded, bool inverse, bool check_done);
@@ -199,7 +214,5 @@ const char* last_launch_failure();
 // Record the CUDA error behind an SCFFT_ECUDA for scfft_last_cuda_error() (defined in capi.cu).
 void note_cuda_error(cudaError_t e, const char* file, int line);
 
-FftPlan make_plan(int L);
-bool length_supported(int L);
 
 }  // namespace scfft

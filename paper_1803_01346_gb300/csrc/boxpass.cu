@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(kBoxThreads, 1) boxpass_kernel(const BoxArgs a
   constexpr int R1p = S::R1p, R2p = S::R2p, TC3 = S::TC3, S2p = S::S2p;
   constexpr int HXu = S::HXu, HXp = S::HXp;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   float2* ty = sm;              // [N]       W_N^m
@@ -350,7 +351,7 @@ template <int N> cudaError_t go_box(const Launch<float>& L, bool chk) {
   a.offS = P.offS;
   a.offB = P.offB;
   const dim3 grid(3 * (L.bz1 - L.bz0));  // one CTA per (component, plane of the box)
-  k<<<grid, kBoxThreads, P.smem, L.st>>>(a);
+  launch_chained(k, dim3(grid), kBoxThreads, P.smem, L.st, a);
   return checked_launch("boxpass_kernel", grid, kBoxThreads, P.smem);
 }
 

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
   constexpr int NL = HALF ? R2 / 2 : R2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int unit[TC];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   int4* tw = reinterpret_cast<int4*>(smem_raw);
   fxc* sm = reinterpret_cast<fxc*>(tw + L);
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
   constexpr int CS = cmax(R2 * S2, R1 * S1);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int unit[6][TC];  // units of the three spectra, of the three products' transforms
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   int4* tw = reinterpret_cast<int4*>(smem_raw);
   fxc* F = reinterpret_cast<fxc*>(tw + L);
@@ -374,6 +376,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
   constexpr int TP = S::TP, P = S::P, NT = S::NT, XL = S::XL, TT = S::TT, Li = S::Li, Lo = S::Lo, R1o = S::R1o;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   int4* twi = reinterpret_cast<int4*>(smem_raw);  // [k2][n1]: the lanes of a pair read consecutive words
   int4* two = twi + S::TWI;
@@ -584,7 +587,7 @@ cudaError_t go_x(const Launch<double>& L, const XArgs<double>& a) {
   const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P;
   const int grid = ntiles < resident ? ntiles : resident;
   const Work<double>& w = *L.w;
-  k<<<grid, S::NT, smem, L.st>>>(a, CIN == 2 ? w.fxp[0] : w.fxu[0], COUT == 2 ? w.fxp[0] : w.fxu[0]);
+  launch_chained(k, dim3(grid), S::NT, smem, L.st, a, CIN == 2 ? w.fxp[0] : w.fxu[0], COUT == 2 ? w.fxp[0] : w.fxu[0]);
   return checked_launch("fx xpass_kernel", dim3(grid), S::NT, smem);
 }
 template <int CIN, int COUT> cudaError_t go_x_n(const Launch<double>& L, const XArgs<double>& a) {

@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_reg_kernel(typename cplx_of<T>:
   constexpr int L = R1 * R2;
   constexpr int S2 = R1 * TC + kPad8;  // transpose row stride
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (check_done && ctrl->done) return;
   V* tw = reinterpret_cast<V*>(smem_raw);
   V* sm = tw + L;
@@ -220,7 +221,7 @@ cudaError_t go_y(const Launch<float>& L, float2* base, int rows, int sx, int HX,
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return per_sm > 0 && sms > 0 ? per_sm * sms : 0;
   }();
-  k<<<grid, TC * R1, smem, L.st>>>(base, rows, sx, HX, L.g.nz, tw, L.ctrl, chk ? 1 : 0, resident, box ? L.bz0 : 0,
+  launch_chained(k, dim3(grid), TC * R1, smem, L.st, base, rows, sx, HX, L.g.nz, tw, L.ctrl, chk ? 1 : 0, resident, box ? L.bz0 : 0,
                                    box ? L.by0 : 0, box ? L.by1 : rows);
   return cudaGetLastError();
 }
@@ -243,7 +244,7 @@ cudaError_t go_z(const Launch<float>& L, float2* base, int rows, int sx, int HX,
   const Work<float>& w = *L.w;
   // box: the padded pass's input planes, or the curl pass's output planes (both Omega's box)
   const bool box = L.use_box;
-  k<<<grid, TC * R1, smem, L.st>>>(base, rows, sx, HX, L.g.nz, tw, w.kt[0], w.kt[1], w.kt[2], w.st[0], w.st[1],
+  launch_chained(k, dim3(grid), TC * R1, smem, L.st, base, rows, sx, HX, L.g.nz, tw, w.kt[0], w.kt[1], w.kt[2], w.st[0], w.st[1],
                                    w.st[2], (float)scale, w.kap4, L.g.nx, L.g.ny, L.g.nz, L.ctrl, chk ? 1 : 0,
                                    box ? L.bz0 : 0, box ? L.bz1 : Lt);
   return cudaGetLastError();
@@ -261,7 +262,7 @@ template <int TC> cudaError_t go_z_tm2(const Launch<float>& L, bool chk) {
   const int nfull = HX / TC, rem = HX - nfull * TC;
   const dim3 grid(nfull * rows + (rows * rem + TC - 1) / TC, 1, 1);
   const bool box = L.use_box;
-  k<<<grid, TC * 16, smem, L.st>>>(L.w->Pd, rows, g.sxp, HX, g.nz, L.w->twp[2], L.w->kap4, g.nx, g.ny, g.nz, L.ctrl,
+  launch_chained(k, dim3(grid), TC * 16, smem, L.st, L.w->Pd, rows, g.sxp, HX, g.nz, L.w->twp[2], L.w->kap4, g.nx, g.ny, g.nz, L.ctrl,
                                    chk ? 1 : 0, box ? L.bz0 : 0, box ? L.bz1 : Lt);
   return checked_launch("zpass_tm2_kernel", grid, TC * 16, smem);
 }
@@ -489,7 +490,7 @@ cudaError_t go_x(const XRArgs& a, cudaStream_t st) {
     return per_sm > 0 && sms > 0 ? per_sm * sms : 1024;
   }();
   const int grid = ntiles < resident ? ntiles : resident;
-  k<<<grid, kPairs * S::TP, smem, st>>>(a);
+  launch_chained(k, dim3(grid), kPairs * S::TP, smem, st, a);
   return checked_launch("xpass_reg2_kernel", dim3(grid), kPairs * S::TP, smem);
 }
 
@@ -513,7 +514,7 @@ cudaError_t go_xu3(const XRArgs& a, cudaStream_t st) {
     return per_sm > 0 && sms > 0 ? per_sm * sms : 1024;
   }();
   const int grid = ntiles < resident ? ntiles : resident;
-  k<<<grid, NT, smem, st>>>(a);
+  launch_chained(k, dim3(grid), NT, smem, st, a);
   return checked_launch("xupdate3_kernel", dim3(grid), NT, smem);
 }
 
@@ -639,6 +640,7 @@ __global__ void __launch_bounds__(TC * R1, (R1 == R2 && KIND >= 1) ? 4 : 1) zpas
   constexpr int CS = OWN ? cmax(R2 * S2, R1 * S1) : cmax(cmax(R2 * S2, R1 * S1), L * TC);
   constexpr int NT = TC * R1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (check_done && ctrl->done) return;
   float2* tw = reinterpret_cast<float2*>(smem_raw);
   float2* F = tw + L;
@@ -987,6 +989,7 @@ __global__ void __launch_bounds__(TC * 16, 6)
   constexpr int CS = R * S2;          // one buffer
   constexpr int NT = TC * R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (check_done && ctrl->done) return;
   float2* tw = reinterpret_cast<float2*>(smem_raw);
   float2* FA = tw + L;
@@ -1203,6 +1206,7 @@ __global__ void __launch_bounds__(P * XS<MODE, R1i, R2i, R2o>::TP, 4)
   constexpr int XL = S::C2R ? (S::PADIN ? Li / 2 : Li) : (S::PADOUT ? Lo / 2 : Lo);  // nx
   constexpr int TT = cmax(cmax(S::C2R ? R2i * (R1i + 1) : 1, S::R2C ? R2o * (R1o + 1) : 1), S::R2C ? Lo : 1);
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   // The update pass takes the iteration index from the device (Ctrl::iters, advanced by its
   // own last CTA) and dh_e/dt, the stop threshold and 1/|Omega_out| from the device copy of
@@ -1586,6 +1590,7 @@ __global__ void __launch_bounds__(3 * P * XS<X_UPDATE, R1i, R2i, R2o>::TP, 16 / 
   constexpr int TT = cmax(cmax(R2i * (R1i + 1), R2o * (R1o + 1)), Lo);
   constexpr int J = XL / TP;    // node pairs of a lane
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   const int it = *reinterpret_cast<volatile const int*>(&a.ctrl->iters);
   const float* h_old = a.hbuf[it & 1];

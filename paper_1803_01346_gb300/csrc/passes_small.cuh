@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(96) xpass_kernel(const XArgs<double> a) {
   typedef Lanes<Lo> FO;
   __shared__ __align__(16) double2 RS[CIN ? 3 : 1][CIN ? NX : 1];       // real rows of the pair, as complex values
   __shared__ __align__(16) double2 Z[COUT ? 3 : 1][COUT ? Lo : 1];
+  after_previous();
   const int done = a.check_done ? a.ctrl->done : 0;  // (looked at once the input is on its way)
   const int t = threadIdx.x, lane = t & 31, q = t >> 5;
   const int ny = a.g.ny, nz = a.g.nz;
@@ -268,6 +269,7 @@ struct YArgs {
 // 16 and 32 points: one warp a CTA, two or one columns (component, plane, kx).
 template <int L, bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass_lanes_kernel(const YArgs a) {
   constexpr int C = 32 / L, SH = C == 2 ? 1 : 0;
+  after_previous();
   const int done = a.check_done ? a.ctrl->done : 0;
   const int c = threadIdx.x % C, row = threadIdx.x / C;
   const int i = blockIdx.x * C + c;
@@ -288,6 +290,7 @@ template <bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass64_kern
   constexpr int L = 64, TC = 4;
   constexpr bool HALF = PAD && !INV;
   __shared__ __align__(16) double2 tw[L], T[L * TC];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   const int t = threadIdx.x, c = t % TC, n1 = t / TC;
   const int e = blockIdx.x * TC + c;
@@ -332,6 +335,7 @@ template <int L, int KIND> __global__ void __launch_bounds__(96) zpass_lanes_ker
   constexpr int C = 32 / L, SH = C == 2 ? 1 : 0;
   constexpr bool PR = KIND == 1;
   __shared__ __align__(16) double2 F[3][32];
+  after_previous();
   const int done = a.check_done ? a.ctrl->done : 0;
   const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
   const int c = lane % C, l = lane / C;
@@ -375,6 +379,7 @@ template <int L, int KIND> __global__ void __launch_bounds__(96) zpass_lanes_ker
 __global__ void __launch_bounds__(96) zpass64_kernel(const ZArgs a) {
   constexpr int L = 64, TC = 4, NT = 96;
   __shared__ __align__(16) double2 tw[L], T[3][L * TC], F[3][L * TC];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   const int t = threadIdx.x, c = t % TC, n1 = (t / TC) % 8, q = t / (TC * 8);
   const int ncol = a.rows * a.HX;

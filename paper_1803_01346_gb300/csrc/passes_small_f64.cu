@@ -6,8 +6,8 @@ namespace small {
 
 template <int CIN, int COUT> static cudaError_t go_x(const XArgs<double>& a, cudaStream_t st) {
   const int grid = (a.use_box ? a.bz1 - a.bz0 : a.g.nz) * ((a.use_box ? a.by1 - a.by0 : a.g.ny) / 2);
-  if (a.g.nx == 16) xpass_kernel<CIN, COUT, 16><<<grid, 96, 0, st>>>(a);
-  else if (a.g.nx == 32) xpass_kernel<CIN, COUT, 32><<<grid, 96, 0, st>>>(a);
+  if (a.g.nx == 16) launch_chained(xpass_kernel<CIN, COUT, 16>, dim3(grid), 96, 0, st, a);
+  else if (a.g.nx == 32) launch_chained(xpass_kernel<CIN, COUT, 32>, dim3(grid), 96, 0, st, a);
   else return cudaErrorInvalidValue;
   return checked_launch("small xpass_kernel", dim3(grid), 96, 0);
 }
@@ -28,8 +28,8 @@ cudaError_t launch_x(const XArgs<double>& a, int cin, int cout, cudaStream_t st)
 template <int L, bool INV, bool PAD> static cudaError_t go_y(const YArgs& a, cudaStream_t st) {
   constexpr int tc = L == 64 ? 4 : 32 / L;
   const int grid = (3 * a.planes * a.HX + tc - 1) / tc;
-  if constexpr (L == 64) ypass64_kernel<INV, PAD><<<grid, 32, 0, st>>>(a);
-  else ypass_lanes_kernel<L, INV, PAD><<<grid, 32, 0, st>>>(a);
+  if constexpr (L == 64) launch_chained(ypass64_kernel<INV, PAD>, dim3(grid), 32, 0, st, a);
+  else launch_chained(ypass_lanes_kernel<L, INV, PAD>, dim3(grid), 32, 0, st, a);
   return checked_launch("small y pass", dim3(grid), 32, 0);
 }
 
@@ -63,8 +63,8 @@ cudaError_t launch_y(const Launch<double>& L, bool padded, bool inverse, bool ch
 template <int L, int KIND> static cudaError_t go_z(const ZArgs& a, cudaStream_t st) {
   constexpr int tc = L == 64 ? 4 : 32 / L;
   const int grid = (a.rows * a.HX + tc - 1) / tc;
-  if constexpr (L == 64) zpass64_kernel<<<grid, 96, 0, st>>>(a);
-  else zpass_lanes_kernel<L, KIND><<<grid, 96, 0, st>>>(a);
+  if constexpr (L == 64) launch_chained(zpass64_kernel, dim3(grid), 96, 0, st, a);
+  else launch_chained(zpass_lanes_kernel<L, KIND>, dim3(grid), 96, 0, st, a);
   return checked_launch("small z pass", dim3(grid), 96, 0);
 }
 

@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
   constexpr int TP = S::TP, P = S::P, NT = S::NT, XL = S::XL, TT = S::TT, Li = S::Li, Lo = S::Lo, R1o = S::R1o;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   if (a.check_done && a.ctrl->done) return;
   V* twi = reinterpret_cast<V*>(smem_raw);  // [k2][n1]: the lanes of a pair read consecutive words
   V* two = twi + S::TWI;
@@ -435,7 +436,7 @@ cudaError_t go_x(const XArgs<T>& a, cudaStream_t st) {
   const int hp = (a.use_box ? a.by1 - a.by0 : a.g.ny) / 2;
   const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P;
   const int grid = ntiles < resident ? ntiles : resident;
-  k<<<grid, S::NT, smem, st>>>(a);
+  launch_chained(k, dim3(grid), S::NT, smem, st, a);
   return checked_launch("xwide_kernel", dim3(grid), S::NT, smem);
 }
 

@@ -11,7 +11,7 @@ template <int R1, int R2, bool INV, bool PAD> cudaError_t go_y(const Launch<doub
   const size_t smem = sizeof(fxc) * (R1 * R2 + R2 * (R1 * TC + (TC < 8 ? TC : 0)));
   allow_smem<k>();
   const dim3 grid((a.HX + TC - 1) / TC, planes, 3);
-  k<<<grid, TC * R1, smem, L.st>>>(a);
+  launch_chained(k, dim3(grid), TC * R1, smem, L.st, a);
   return checked_launch("fx ypass_kernel", grid, TC * R1, smem);
 }
 template <int R1, int R2, int KIND> cudaError_t go_z(const Launch<double>& L, const ZArgs& a) {
@@ -23,7 +23,7 @@ template <int R1, int R2, int KIND> cudaError_t go_z(const Launch<double>& L, co
   allow_smem<k>();
   const int nfull = a.HX / TC, rem = a.HX - nfull * TC;
   const dim3 grid(nfull * a.rows + (a.rows * rem + TC - 1) / TC);
-  k<<<grid, TC * R1, smem, L.st>>>(a);
+  launch_chained(k, dim3(grid), TC * R1, smem, L.st, a);
   return checked_launch("fx zpass_kernel", grid, TC * R1, smem);
 }
 

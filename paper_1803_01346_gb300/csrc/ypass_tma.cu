@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_tma_kernel(const __grid_constan
   typedef YT<R1, R2, TC, PIN> S;
   constexpr int L = S::L, SB = S::SB, SBX = S::SBX, S2 = S::S2, NT = TC * R1;
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  after_previous();
   if (check_done && ctrl->done) return;
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);         // [2]
   float2* stage = reinterpret_cast<float2*>(smem_raw + 128);      // [2][SBX], 128-byte aligned
@@ -182,7 +183,7 @@ cudaError_t go_y_tma(const Launch<float>& L, const CUtensorMap& map, float2* bas
   const int grid = ntiles < resident ? ntiles : resident;
   const int inject = (L.fault && *L.fault == SCFFT_FAULT_TMA_WAIT) ? 1 : 0;
   if (inject) *L.fault = 0;  // one shot
-  k<<<grid, TC * R1, S::smem, L.st>>>(map, base, rows, sx, HX, L.g.nz, tw, L.ctrl, chk ? 1 : 0, inject,
+  launch_chained(k, dim3(grid), TC * R1, S::smem, L.st, map, base, rows, sx, HX, L.g.nz, tw, L.ctrl, chk ? 1 : 0, inject,
                                       box ? L.bz0 : 0, nzp, box ? L.by0 : 0, box ? L.by1 : rows);
   return cudaGetLastError();
 }

@@ -46,7 +46,7 @@ struct scfft_ctx {
   cudaGraphExec_t loop_exec = nullptr;
   bool loop_failed = false;
   int fault = 0;  // armed fault injection (scfft_inject_fault)
-  // FP32 path: Ctrl::iter_total already folded into stats, and whether graph-run rhs calls
+  // Ctrl::iter_total already folded into stats, and whether graph-run rhs calls
   // of the integrator have not been folded in yet (their statistics are read once per step)
   unsigned long long iters_seen = 0;
   bool graph_pending = false;
@@ -421,7 +421,7 @@ template <typename T> cudaError_t iteration(scfft_ctx* c, const Launch<T>& L, Po
 }
 
 // ---------------------------------------------------------------- Eq. 5 loop as a CUDA graph
-// The FP32 path runs the whole Eq. 5 iteration loop of one rhs as one graph launch: a WHILE
+// The whole Eq. 5 iteration loop of one rhs runs as one graph launch: a WHILE
 // conditional node whose body is one iteration (the eight passes) followed by a one-thread
 // kernel that sets the loop condition from the device flags (stop reached, status,
 // iteration cap).  No iteration is queued past convergence and the host takes no part
@@ -439,31 +439,35 @@ constexpr int kLoopLaunches = 9;    // kernels per iteration of the graph body
 constexpr int kLoopLaunchesBox = 7; // the same with the fused box passes
 constexpr int kLoopLaunchesFd = 7;  // the same with the local-stencil curl
 
-cudaError_t loop_body(const Launch<float>& L, const PointParams& pp, cudaGraphConditionalHandle h, int max_iter,
+template <typename T>
+cudaError_t loop_body(const Launch<T>& L, const PointParams& pp, cudaGraphConditionalHandle h, int max_iter,
                       bool fd, const double* dcell) {
   cudaError_t e;
   bool fused = false;
   if (fd) {
-    if ((e = launch_fd_curl_mask<float>(L, L.w->Jd, dcell, false)) != cudaSuccess) return e;
-    if ((e = launch_x_reg_io(L, X_PAD_F64, pp, nullptr, L.w->Jd, nullptr, nullptr, nullptr, 0, 0, false)) !=
-        cudaSuccess)
-      return e;
+    if ((e = launch_fd_curl_mask<T>(L, L.w->Jd, dcell, false)) != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4)
+      e = launch_x_reg_io(L, X_PAD_F64, pp, nullptr, L.w->Jd, nullptr, nullptr, nullptr, 0, 0, false);
+    else
+      e = launch_x_pad_rows<T>(L, pp, L.w->Jd, false);
+    if (e != cudaSuccess) return e;
   } else {
-    if ((e = launch_y<float>(L, false, false, false)) != cudaSuccess) return e;
-    if ((e = launch_z_curl<float>(boxed(L), false, 1.0 / (double)L.g.N)) != cudaSuccess) return e;
-    fused = box_fused_on(boxed(L));
-    if (fused) {
-      if ((e = launch_box_fused(boxed(L), false)) != cudaSuccess) return e;
-    } else {
-      if ((e = launch_y<float>(boxed(L), false, true, false)) != cudaSuccess) return e;
-      if ((e = launch_x<float>(boxed(L), X_MASKPAD, pp, nullptr, nullptr, nullptr, 0, 0, false)) != cudaSuccess)
+    if ((e = launch_y<T>(L, false, false, false)) != cudaSuccess) return e;
+    if ((e = launch_z_curl<T>(boxed(L), false, 1.0 / (double)L.g.N)) != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+      fused = box_fused_on(boxed(L));
+      if (fused && (e = launch_box_fused(boxed(L), false)) != cudaSuccess) return e;
+    }
+    if (!fused) {
+      if ((e = launch_y<T>(boxed(L), false, true, false)) != cudaSuccess) return e;
+      if ((e = launch_x<T>(boxed(L), X_MASKPAD, pp, nullptr, nullptr, nullptr, 0, 0, false)) != cudaSuccess)
         return e;
     }
   }
-  if (!fused && (e = launch_y<float>(boxed(L), true, false, false)) != cudaSuccess) return e;
-  if ((e = launch_z_kernel<float>(boxed(L), false)) != cudaSuccess) return e;
-  if ((e = launch_y<float>(L, true, true, false)) != cudaSuccess) return e;
-  if ((e = launch_x<float>(L, fd ? X_UPDATE_FD : X_UPDATE, pp, nullptr, nullptr, nullptr, 0, 1, false)) != cudaSuccess)
+  if (!fused && (e = launch_y<T>(boxed(L), true, false, false)) != cudaSuccess) return e;
+  if ((e = launch_z_kernel<T>(boxed(L), false)) != cudaSuccess) return e;
+  if ((e = launch_y<T>(L, true, true, false)) != cudaSuccess) return e;
+  if ((e = launch_x<T>(L, fd ? X_UPDATE_FD : X_UPDATE, pp, nullptr, nullptr, nullptr, 0, 1, false)) != cudaSuccess)
     return e;
   loop_cond_kernel<<<1, 1, 0, L.st>>>(h, L.ctrl, max_iter);
   return cudaGetLastError();
@@ -471,7 +475,7 @@ cudaError_t loop_body(const Launch<float>& L, const PointParams& pp, cudaGraphCo
 
 // Build the loop graph once per context; false (and the host-driven loop) if the driver
 // refuses any step.
-bool loop_graph_ready(scfft_ctx* c) {
+template <typename T> bool loop_graph_ready(scfft_ctx* c) {
   if (c->loop_exec) return true;
   if (c->loop_failed) return false;
   c->loop_failed = true;  // until the build succeeds
@@ -482,7 +486,7 @@ bool loop_graph_ready(scfft_ctx* c) {
     cudaGetLastError();
     return false;
   }
-  Launch<float> L = launch_of<float>(c);
+  Launch<T> L = launch_of<T>(c);
   L.st = cs;
   L.fault = nullptr;  // a fault is never captured into the loop graph
   const PointParams pp = base_params(c);
@@ -505,7 +509,7 @@ bool loop_graph_ready(scfft_ctx* c) {
     ok = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) == cudaSuccess;
     if (ok) {
       const bool launched =
-          loop_body(L, pp, h, c->opt.max_iter, c->curl_kind == SCFFT_CURL_FD, c->dcell) == cudaSuccess;
+          loop_body<T>(L, pp, h, c->opt.max_iter, c->curl_kind == SCFFT_CURL_FD, c->dcell) == cudaSuccess;
       cudaGraph_t captured = nullptr;
       ok = cudaStreamEndCapture(cs, &captured) == cudaSuccess && launched;
     }
@@ -550,16 +554,17 @@ cudaError_t x_io(const Launch<T>& L, XMode mode, const PointParams& pp, const Rh
     return launch_x<T>(L, mode, pp, io.h64, nullptr, io.warm64, 0, 0, false);
 }
 
-// FP32 path: fold the device's iteration counter into the host statistics (graph-run
+// Fold the device's iteration counter into the host statistics (graph-run
 // iterations also count their kLoopLaunches kernels here).
 void absorb_ctrl(scfft_ctx* c, const Ctrl& hc, bool graph_iters) {
   const unsigned long long d = hc.iter_total - c->iters_seen;
   c->iters_seen = hc.iter_total;
   c->stats.iterations += (long long)d;
   if (graph_iters)
-    c->stats.launches += (long long)(c->curl_kind == SCFFT_CURL_FD     ? kLoopLaunchesFd
-                                     : box_fused_on(boxed(launch_of<float>(c))) ? kLoopLaunchesBox
-                                                                                : kLoopLaunches) *
+    c->stats.launches += (long long)(c->curl_kind == SCFFT_CURL_FD ? kLoopLaunchesFd
+                                     : c->opt.precision == SCFFT_PREC_F32 && box_fused_on(boxed(launch_of<float>(c)))
+                                         ? kLoopLaunchesBox
+                                         : kLoopLaunches) *
                          (long long)d;
   c->stats.last_iters = hc.iters;
   c->stats.last_residual = hc.residual;
@@ -577,13 +582,11 @@ scfft_status flush_pending(scfft_ctx* c) {
   return (scfft_status)hc.status;
 }
 
-// defer (the FP32 integrator's stages): when the loop runs as a graph and the caller wants
+// defer (the integrator's stages): when the loop runs as a graph and the caller wants
 // no iteration count, return without reading the device state back; the step reads it once.
 template <typename T>
 scfft_status rhs_impl(scfft_ctx* c, double t, int left, const RhsIO& io, int* iters_out, bool defer = false) {
-  if constexpr (sizeof(T) == 4) {
-    if (c->graph_pending && !(defer && !iters_out && !c->prof_on)) CS_(flush_pending(c));
-  }
+  if (c->graph_pending && !(defer && !iters_out && !c->prof_on)) CS_(flush_pending(c));
   Launch<T> L = launch_of<T>(c);
   PointParams pp = base_params(c);
   hedot_at(c, t, left, pp.hedot);
@@ -617,11 +620,10 @@ scfft_status rhs_impl(scfft_ctx* c, double t, int left, const RhsIO& io, int* it
   const bool early = c->opt.delta_it > 0 && c->nout > 0;
   int launched = 0;
   bool graphed = false;
-  if constexpr (sizeof(T) == 4) {
-    if (c->nout > 0 && maxit > 0 && !c->prof_on && loop_graph_ready(c)) {
-      CK(cudaGraphLaunch(c->loop_exec, c->st));
-      graphed = true;
-    }
+  // (FP64 at a fixed iteration count: queued by the host, so that the call need not wait for the device)
+  if (c->nout > 0 && maxit > 0 && !c->prof_on && (sizeof(T) == 4 || early) && loop_graph_ready<T>(c)) {
+    CK(cudaGraphLaunch(c->loop_exec, c->st));
+    graphed = true;
   }
   if (c->nout > 0 && !graphed) {
     // With an early stop the host keeps one iteration queued ahead: before
@@ -668,13 +670,7 @@ scfft_status rhs_impl(scfft_ctx* c, double t, int left, const RhsIO& io, int* it
     CK(cudaMemcpyAsync(c->hctrl + 2, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
     const Ctrl hc = c->hctrl[2];
-    if constexpr (sizeof(T) == 4) {
-      absorb_ctrl(c, hc, graphed);
-    } else {
-      c->stats.iterations += hc.iters;
-      c->stats.last_iters = hc.iters;
-      c->stats.last_residual = hc.residual;
-    }
+    absorb_ctrl(c, hc, graphed);
     if (iters_out) *iters_out = hc.iters;
     if (hc.status != 0) return (scfft_status)hc.status;
     if (iters_out && c->nout > 0 && maxit > 0 && !(hc.residual < pp.tol) && c->opt.delta_it > 0)
@@ -682,18 +678,19 @@ scfft_status rhs_impl(scfft_ctx* c, double t, int left, const RhsIO& io, int* it
   } else {
     c->stats.iterations += launched;
     c->stats.last_iters = launched;
-    if constexpr (sizeof(T) == 4) c->iters_seen += (unsigned long long)launched;  // no early stop: all ran
+    c->iters_seen += (unsigned long long)launched;  // no early stop: all ran
   }
   return SCFFT_OK;
 }
 
-scfft_status rhs_any(scfft_ctx* c, double t, int left, const double* h, double* warm, double* hdot, int* it) {
+scfft_status rhs_any(scfft_ctx* c, double t, int left, const double* h, double* warm, double* hdot, int* it,
+                     bool defer = false) {
   RhsIO io;
   io.h64 = h;
   io.warm64 = warm;
   io.out64 = hdot;
   io.warm_out64 = warm;
-  return by_prec(c, [&](auto z) { return rhs_impl<decltype(z)>(c, t, left, io, it); });
+  return by_prec(c, [&](auto z) { return rhs_impl<decltype(z)>(c, t, left, io, it, defer); });
 }
 
 template <typename T> scfft_status curl_impl(scfft_ctx* c, const double* f, double* out) {
@@ -806,17 +803,17 @@ scfft_status bs23_step(scfft_ctx* c, double* t_io, double* dt_io, double tstop, 
       combine_kernel<<<blocks, 256, 0, c->st>>>(ytmp, h, hs, a21, k[0], 0, nullptr, 0, nullptr, n3);
       return cudaGetLastError();
     }));
-    CS_(rhs_any(c, t + 0.5 * hs, 0, ytmp, g, k[1], nullptr));
+    CS_(rhs_any(c, t + 0.5 * hs, 0, ytmp, g, k[1], nullptr, true));
     CK(run(c, SCFFT_K_RK, [&] {
       combine_kernel<<<blocks, 256, 0, c->st>>>(ytmp, h, hs, 0.0, k[0], a32, k[1], 0, nullptr, n3);
       return cudaGetLastError();
     }));
-    CS_(rhs_any(c, t + 0.75 * hs, 0, ytmp, g, k[2], nullptr));
+    CS_(rhs_any(c, t + 0.75 * hs, 0, ytmp, g, k[2], nullptr, true));
     CK(run(c, SCFFT_K_RK, [&] {
       combine_kernel<<<blocks, 256, 0, c->st>>>(ynew, h, hs, b1, k[0], b2, k[1], b3, k[2], n3);
       return cudaGetLastError();
     }));
-    CS_(rhs_any(c, hits ? nxt : t + hs, end_left ? 1 : 0, ynew, g, k[3], nullptr));
+    CS_(rhs_any(c, hits ? nxt : t + hs, end_left ? 1 : 0, ynew, g, k[3], nullptr, true));
     double en = 0.0;
     if (!(dt_fixed > 0)) {
       CK(cudaMemsetAsync(c->errbits, 0, sizeof(unsigned long long), c->st));
@@ -826,12 +823,27 @@ scfft_status bs23_step(scfft_ctx* c, double* t_io, double* dt_io, double tstop, 
         return cudaGetLastError();
       }));
       CK(cudaMemcpyAsync(c->herr, c->errbits, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->st));
-      CK(cudaStreamSynchronize(c->st));
+      if (c->graph_pending) {
+        const scfft_status ds = flush_pending(c);  // synchronises the stream
+        if (ds != SCFFT_OK) {
+          c->fsal_valid = false;
+          return ds;
+        }
+      } else {
+        CK(cudaStreamSynchronize(c->st));
+      }
       const unsigned long long bits = *c->herr;
       memcpy(&en, &bits, sizeof(double));
       if (!(en == en)) {
         c->fsal_valid = false;
         return SCFFT_ENONFINITE;
+      }
+    }
+    if (c->graph_pending) {  // fixed step: no error norm was read, read the device state here
+      const scfft_status ds = flush_pending(c);
+      if (ds != SCFFT_OK) {
+        c->fsal_valid = false;
+        return ds;
       }
     }
     if (en <= 1.0) {
@@ -1317,7 +1329,7 @@ bool capture_eq5_loop(scfft_ctx* c, cudaStream_t cs, cudaStream_t cs2, const Poi
   Launch<float> L2 = launch_of<float>(c);
   L2.st = cs2;
   L2.fault = nullptr;
-  const bool ok = loop_body(L2, pp, hh, c->opt.max_iter, c->curl_kind == SCFFT_CURL_FD, c->dcell) == cudaSuccess;
+  const bool ok = loop_body<float>(L2, pp, hh, c->opt.max_iter, c->curl_kind == SCFFT_CURL_FD, c->dcell) == cudaSuccess;
   cudaGraph_t captured = nullptr;
   return cudaStreamEndCapture(cs2, &captured) == cudaSuccess && ok;
 }

@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   after_previous();
   if (a.check_done && a.ctrl->done) return;
+  const UpdateArgs<double> up = update_args(a);
   int4* twi = reinterpret_cast<int4*>(smem_raw);  // [k2][n1]: the lanes of a pair read consecutive words
   int4* two = twi + S::TWI;
   double2* RS = reinterpret_cast<double2*>(two + S::TWO);  // [3][P][XL] real rows of the pairs
@@ -461,8 +462,8 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
 #pragma unroll
         for (int q = 0; q < 3; ++q) w[q] = RS[(q * P + p) * XL + x];
         double va[3] = {w[0].x, w[1].x, w[2].x}, vb[3] = {w[0].y, w[1].y, w[2].y};
-        part += node_step<double>(a, na0 + x, va);
-        part += node_step<double>(a, na0 + XL + x, vb);
+        part += node_step<double>(a, up, na0 + x, va);
+        part += node_step<double>(a, up, na0 + XL + x, vb);
         if (COUT > 0) {
 #pragma unroll
           for (int q = 0; q < 3; ++q) RS[(q * P + p) * XL + x] = make_double2(va[q], vb[q]);
@@ -571,8 +572,8 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
     }
     __syncwarp();  // the pair's rows are reused by the next tile
   }
-  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<NT>(a, part);
-  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && tid == 0) reset_ctrl(a.ctrl);
+  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<NT>(a, part, up.it);
+  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && tid == 0) begin_loop(a);
 }
 
 // ---------------------------------------------------------------- launchers

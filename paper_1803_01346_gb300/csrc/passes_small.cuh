@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(96) xpass_kernel(const XArgs<double> a) {
   __shared__ __align__(16) double2 Z[COUT ? 3 : 1][COUT ? Lo : 1];
   after_previous();
   const int done = a.check_done ? a.ctrl->done : 0;  // (looked at once the input is on its way)
+  const UpdateArgs<double> up = update_args(a);
   const int t = threadIdx.x, lane = t & 31, q = t >> 5;
   const int ny = a.g.ny, nz = a.g.nz;
   const long long N = a.g.N;
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(96) xpass_kernel(const XArgs<double> a) {
         p[c] = &RS[c][x].x + r;
         w[c] = *p[c];
       }
-      part += node_step<double>(a, na0 + i, w);
+      part += node_step<double>(a, up, na0 + i, w);
       if (COUT > 0) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) *p[c] = w[c];
@@ -234,8 +235,8 @@ __global__ void __launch_bounds__(96) xpass_kernel(const XArgs<double> a) {
           second ? mk((Zk.y + Zm.y) * 0.5, (Zm.x - Zk.x) * 0.5) : mk((Zk.x + Zm.x) * 0.5, (Zk.y - Zm.y) * 0.5);
     }
   }
-  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<96>(a, part);
-  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && t == 0) reset_ctrl(a.ctrl);
+  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<96>(a, part, up.it);
+  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && t == 0) begin_loop(a);
 }
 
 // ---------------------------------------------------------------- 64 points, 8 to a thread

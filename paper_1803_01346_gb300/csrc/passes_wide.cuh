@@ -86,22 +86,40 @@ struct XArgs {
   const double* warm;
   const uint8_t* mask;
   const T* jc;
-  const T* hold;
-  T* hnew;
+  T* hbuf[2];       // both iterate buffers: the update pass picks by the device's iteration count
   PointParams pp;
+  PointParams* ppd; // device copy of pp (written by the assemble pass, read by the update pass)
   Ctrl* ctrl;
   double* partials;
   int check_done;
-  int out_buf;
   // mask/pad pass of an Eq. 5 iteration: only the rows of Omega's box (y in [by0, by1), z in
   // [bz0, bz1)); the source vanishes outside, and nothing downstream reads the rows left out
   int use_box, by0, by1, bz0, bz1;
 };
 
+// What the update pass takes from the device, so that a captured launch serves every iteration:
+// its iteration index, the iterate buffers and dh_e/dt.
+template <typename T> struct UpdateArgs {
+  int it = 0;
+  const T* hold = nullptr;
+  T* hnew = nullptr;
+  T hedot[3];
+};
+template <typename T> __device__ __forceinline__ UpdateArgs<T> update_args(const XArgs<T>& a) {
+  UpdateArgs<T> u;
+  if (a.mode == X_UPDATE) {
+    u.it = *reinterpret_cast<volatile const int*>(&a.ctrl->iters);  // (residual_finish writes it at the end)
+    u.hold = (u.it & 1) ? a.hbuf[1] : a.hbuf[0];
+    u.hnew = (u.it & 1) ? a.hbuf[0] : a.hbuf[1];
+    for (int q = 0; q < 3; ++q) u.hedot[q] = (T)a.ppd->hedot[q];
+  }
+  return u;
+}
+
 // The node-wise step of an x pass on one node's three real values v (in and out); returns the
 // node's summand of the Eq. 5 residual (the update modes, 0 otherwise).
 template <typename T>
-__device__ __forceinline__ double node_step(const XArgs<T>& a, size_t node, T v[3]) {
+__device__ __forceinline__ double node_step(const XArgs<T>& a, const UpdateArgs<T>& up, size_t node, T v[3]) {
   typedef T A;
   const PointParams& pp = a.pp;
   const long long N = a.g.N;
@@ -140,22 +158,22 @@ __device__ __forceinline__ double node_step(const XArgs<T>& a, size_t node, T v[
       } else {
         v[0] = (T)a.warm[node]; v[1] = (T)a.warm[N + node]; v[2] = (T)a.warm[2 * N + node];
       }
-      a.hnew[node] = v[0]; a.hnew[N + node] = v[1]; a.hnew[2 * N + node] = v[2];
+      a.hbuf[0][node] = v[0]; a.hbuf[0][N + node] = v[1]; a.hbuf[0][2 * N + node] = v[2];
       return 0.0;
     case X_MASKPAD:
     case X_ADJ_CROP:
       if (!a.mask[node]) { v[0] = 0; v[1] = 0; v[2] = 0; }
       return 0.0;
     case X_UPDATE: {
-      const T o0 = a.hold[node], o1 = a.hold[N + node], o2 = a.hold[2 * N + node];
+      const T o0 = up.hold[node], o1 = up.hold[N + node], o2 = up.hold[2 * N + node];
       double d = 0.0;
       if (a.mask[node]) {
         v[0] = o0; v[1] = o1; v[2] = o2;
       } else {
-        v[0] = (T)pp.hedot[0] + v[0]; v[1] = (T)pp.hedot[1] + v[1]; v[2] = (T)pp.hedot[2] + v[2];
+        v[0] = up.hedot[0] + v[0]; v[1] = up.hedot[1] + v[1]; v[2] = up.hedot[2] + v[2];
         d = dnorm3(v[0], o0, v[1], o1, v[2], o2);
       }
-      a.hnew[node] = v[0]; a.hnew[N + node] = v[1]; a.hnew[2 * N + node] = v[2];
+      up.hnew[node] = v[0]; up.hnew[N + node] = v[1]; up.hnew[2 * N + node] = v[2];
       return d;
     }
     case X_TO_F64:
@@ -197,7 +215,7 @@ __device__ __forceinline__ double node_step(const XArgs<T>& a, size_t node, T v[
 
 // The end of an Eq. 5 update pass: the deterministic two-level reduction of the residual's
 // summands, the stop flag and the iterate's bookkeeping (written by the last CTA).
-template <int NT, typename T> __device__ void residual_finish(const XArgs<T>& a, double part) {
+template <int NT, typename T> __device__ void residual_finish(const XArgs<T>& a, double part, int it) {
   __shared__ double red[NT / 32];
   __shared__ int am_last;
   const int tid = threadIdx.x;
@@ -224,18 +242,22 @@ template <int NT, typename T> __device__ void residual_finish(const XArgs<T>& a,
   if (tid == 0) {
     double tot = 0.0;
     for (int i = 0; i < NT / 32; ++i) tot += red[i];
-    const double res = tot * a.pp.inv_nout;
+    const double res = tot * a.ppd->inv_nout;
     Ctrl* c = a.ctrl;
     c->residual = res;
-    c->iters = a.pp.iter + 1;
-    c->cur = a.out_buf;
+    c->iters = it + 1;
+    c->iter_total += 1;
+    c->cur = (it + 1) & 1;
     const bool finite = isfinite(res);
     if (!finite) c->status = 6;  // SCFFT_ENONFINITE
-    c->done = (!finite || res < a.pp.tol) ? 1 : 0;
+    c->done = (!finite || res < a.ppd->tol) ? 1 : 0;
     c->counter = 0;
   }
 }
-__device__ __forceinline__ void reset_ctrl(Ctrl* c) {
+template <typename T> __device__ __forceinline__ void begin_loop(const XArgs<T>& a) {
+  *a.ppd = a.pp;
+  Ctrl* c = a.ctrl;
+  c->trips = 0;
   c->done = 0;
   c->iters = 0;
   c->cur = 0;
@@ -270,6 +292,7 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   after_previous();
   if (a.check_done && a.ctrl->done) return;
+  const UpdateArgs<T> up = update_args(a);
   V* twi = reinterpret_cast<V*>(smem_raw);  // [k2][n1]: the lanes of a pair read consecutive words
   V* two = twi + S::TWI;
   V* RS = two + S::TWO;  // [3][P][XL] real rows of the pairs, as complex values
@@ -335,8 +358,8 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) u[q] = RS[(q * P + p) * XL + x];
         T va[3] = {u[0].x, u[1].x, u[2].x}, vb[3] = {u[0].y, u[1].y, u[2].y};
-        part += node_step<T>(a, na0 + x, va);
-        part += node_step<T>(a, na0 + XL + x, vb);
+        part += node_step<T>(a, up, na0 + x, va);
+        part += node_step<T>(a, up, na0 + XL + x, vb);
         if (COUT > 0) {
 #pragma unroll
           for (int q = 0; q < 3; ++q) RS[(q * P + p) * XL + x] = mk(va[q], vb[q]);
@@ -419,8 +442,8 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
     __syncwarp();  // the pair's rows are reused by the next tile
   }
 
-  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<NT>(a, part);
-  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && tid == 0) reset_ctrl(a.ctrl);
+  if (CIN == 2 && a.mode == X_UPDATE) residual_finish<NT>(a, part, up.it);
+  if (CIN == 1 && a.mode == X_ASSEMBLE && blockIdx.x == 0 && tid == 0) begin_loop(a);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -511,13 +534,13 @@ static cudaError_t launch_x_impl(const Launch<T>& L, XMode mode, const PointPara
   a.warm = warm;
   a.mask = L.mask;
   a.jc = L.w->jc;
-  a.hold = L.w->Hd[in_buf];
-  a.hnew = L.w->Hd[out_buf];
+  a.hbuf[0] = L.w->Hd[0];
+  a.hbuf[1] = L.w->Hd[1];
   a.pp = pp;
+  a.ppd = L.ppd;
   a.ctrl = L.ctrl;
   a.partials = L.partials;
   a.check_done = check_done ? 1 : 0;
-  a.out_buf = out_buf;
   a.use_box = (L.use_box && mode == X_MASKPAD) ? 1 : 0;
   a.by0 = L.by0;
   a.by1 = L.by1;

@@ -170,7 +170,7 @@ struct Launch {
 // the start of the next counts.  A pass launched by launch_chained is set up while the kernel before
 // it ends; after_previous, its first statement, holds it until that kernel has ended and its writes are
 // visible.  (Every thread passes through it before the kernel touches memory or returns, so a
-// kernel that has ended implies that all before it have.)  Measured: 16^3 FP64 curl 18.6 -> 12.1 us, Phi
+// kernel that has ended implies that all before it have.)  Measured: 16^3 FP64 curl 22.3 -> 12.1 us, Phi
 // 48 x 32 x 128 FP32 57.1 -> 45.8, reverse mode 48^3 FP64 1251 -> 1109 us.  No pass signals
 // before it ends (griddepcontrol.launch_dependents): the next one's CTAs then fill
 // the SMs that drain first and sit there unevenly (rhs 64 x 64 x 96 FP64 3.55 ms against 3.15 with

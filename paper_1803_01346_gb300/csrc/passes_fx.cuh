@@ -67,7 +67,9 @@ struct YArgs {
   const int4* tw;
   const Ctrl* ctrl;
   int check_done;
-  int zoff, ylo, yhi;  // planes z = zoff + blockIdx.y; input rows outside [ylo, yhi) read as zero
+  // planes z = zoff + blockIdx.y; rows outside [ylo, yhi): the forward pass reads them as zero, the
+  // unpadded inverse pass does not write them
+  int zoff, ylo, yhi;
 };
 
 // grid (ceil(HX / TC), planes, 3), TC columns of one (component, plane) per CTA.  PAD: the
@@ -129,7 +131,10 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
     DFT<R1, INV, fxc>::run(w);
     if (colok) {
 #pragma unroll
-      for (int k1 = 0; k1 < (PAD && INV ? R1 / 2 : R1); ++k1) col[(size_t)(n1 + R2 * k1) * a.sx] = dbl_of(w[k1], U);
+      for (int k1 = 0; k1 < (PAD && INV ? R1 / 2 : R1); ++k1) {
+        const int row = n1 + R2 * k1;
+        if (!INV || PAD || (row >= a.ylo && row < a.yhi)) col[(size_t)row * a.sx] = dbl_of(w[k1], U);
+      }
     }
   }
 }
@@ -151,7 +156,7 @@ struct ZArgs {
   int nx, ny, nz;
   const Ctrl* ctrl;
   int check_done;
-  int zlo, zhi;  // the padded pass's input planes outside [zlo, zhi) read as zero
+  int zlo, zhi;  // planes outside [zlo, zhi): the padded pass reads them as zero, the curl's does not write them
 };
 
 // |c| < 2^dexp(c)
@@ -362,7 +367,10 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
     DFT<R2, true, fxc>::run(v);
     if (colok) {
 #pragma unroll
-      for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) col[q * cstride + (n1 + R1 * m2) * zstride] = dbl_of(v[m2], U);
+      for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) {
+        const int l = n1 + R1 * m2;
+        if (PR || (l >= a.zlo && l < a.zhi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
+      }
     }
   }
 }

@@ -265,7 +265,9 @@ struct YArgs {
   const double2* tw;
   const Ctrl* ctrl;
   int check_done;
-  int zoff, ylo, yhi;  // planes from zoff; input rows outside [ylo, yhi) read as zero (forward)
+  // planes from zoff; rows outside [ylo, yhi): the forward pass reads them as zero, the unpadded
+  // inverse pass does not write them
+  int zoff, ylo, yhi;
 };
 // 16 and 32 points: one warp a CTA, two or one columns (component, plane, kx).
 template <int L, bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass_lanes_kernel(const YArgs a) {
@@ -284,7 +286,7 @@ template <int L, bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass
   if (done) return;
   Lanes<L>::template run<INV, SH>(&v, row, &tw);
   const int o = Lanes<L>::out(row);
-  if (ok && (!(PAD && INV) || o < L / 2)) col[(size_t)o * a.sx] = v;
+  if (ok && (!INV || (PAD ? o < L / 2 : o >= a.ylo && o < a.yhi))) col[(size_t)o * a.sx] = v;
 }
 // 64 points: 32-thread CTAs, 8 threads a column and 8 points a thread.
 template <bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass64_kernel(const YArgs a) {
@@ -328,7 +330,7 @@ struct ZArgs {
   int nx, ny, nz;
   const Ctrl* ctrl;
   int check_done;
-  int zlo, zhi;  // the padded pass's input planes outside [zlo, zhi) read as zero
+  int zlo, zhi;  // planes outside [zlo, zhi): the padded pass reads them as zero, the curl's does not write them
 };
 // 16 and 32 points: one CTA of three warps, a component to a warp, for two or one columns (kx, y);
 // the three spectra meet in shared memory, where each thread takes the product of its own component.
@@ -373,7 +375,7 @@ template <int L, int KIND> __global__ void __launch_bounds__(96) zpass_lanes_ker
   const double2 x = mk(kb * Fc.x - kc * Fb.x, kb * Fc.y - kc * Fb.y);
   v = PR ? mk(-x.y, x.x) : mk(-s * x.y, s * x.x);
   Lanes<L>::template run<true, SH>(&v, l, &tw);
-  if (ok && (!PR || o < L / 2)) col[o * zstride] = v;
+  if (ok && (PR ? o < L / 2 : o >= a.zlo && o < a.zhi)) col[o * zstride] = v;
 }
 // 64 points (always the padded pass): four columns (kx, y) a CTA, its threads over (component,
 // residue, column), 8 points a thread; the product over the spectra in shared memory.

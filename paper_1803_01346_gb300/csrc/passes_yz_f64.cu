@@ -38,8 +38,9 @@ cudaError_t launch_y(const Launch<double>& L, bool padded, bool inverse, bool ch
   a.tw = padded ? L.w->fxp[1] : L.w->fxu[1];
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
-  // the padded forward pass of an Eq. 5 iteration: only the planes and rows of Omega's box
-  const bool box = L.use_box && padded && !inverse;
+  // the padded forward pass and the curl's unpadded inverse pass of an Eq. 5 iteration: only the
+  // planes and rows of Omega's box
+  const bool box = L.use_box && padded != inverse;
   a.zoff = box ? L.bz0 : 0;
   a.ylo = box ? L.by0 : 0;
   a.yhi = box ? L.by1 : a.rows;
@@ -79,8 +80,8 @@ cudaError_t launch_z(const Launch<double>& L, bool padded, bool check_done, doub
   a.nx = g.nx; a.ny = g.ny; a.nz = g.nz;
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
-  a.zlo = (padded && L.use_box) ? L.bz0 : 0;  // the source box of an Eq. 5 iteration
-  a.zhi = (padded && L.use_box) ? L.bz1 : Lz;
+  a.zlo = L.use_box ? L.bz0 : 0;  // the source box of an Eq. 5 iteration
+  a.zhi = L.use_box ? L.bz1 : Lz;
 #define ZCASE_U(LL, R1, R2) case LL: return go_z<R1, R2, 0>(L, a);
 #define ZCASE_P(LL, R1, R2) case LL: return go_z<R1, R2, 1>(L, a);
   if (padded) {

@@ -176,7 +176,7 @@ typedef struct {
  * only when it is more than 3% faster), and caches the choice per device and grid for the
  * process, so that later contexts of that grid (a batch) reuse it without timing; retune != 0
  * times again.  Rebuilds the context's captured graphs on their next launch.  FP64 and
- * double-float contexts have no schedule: SCFFT_OK, nothing timed.  out (may be NULL)
+ * SCFFT_PREC_DF64 contexts have no schedule: SCFFT_OK, nothing timed.  out (may be NULL)
  * receives the schedule in use.  Errors: SCFFT_EINVAL (NULL ctx), SCFFT_ECUDA. */
 scfft_status scfft_autotune(scfft_ctx* ctx, int retune, scfft_schedule* out);
 /* The schedule in use (out->us zero). */

@@ -183,6 +183,13 @@ template <typename T> Launch<T> boxed(const Launch<T>& L) {
   return B;
 }
 
+// The same for the transposed iteration of the reverse mode: its other end is confined to the box.
+template <typename T> Launch<T> tboxed(const Launch<T>& L) {
+  Launch<T> B = L;
+  B.use_tbox = B.by1 > B.by0 && B.bz1 > B.bz0;
+  return B;
+}
+
 // The schedule asks for the fused box passes and they apply to this launch (FP32, nx == ny).
 bool box_fused_on(const Launch<float>& L) { return L.w->sched.box_fused && box_fused_ok(L); }
 
@@ -359,7 +366,8 @@ PointParams base_params(const scfft_ctx* c) {
 }
 
 // ---------------------------------------------------------------- rhs
-// Spectral curl of the half spectrum held in U: y fwd, z (fwd, curl, inv), y inv.
+// Spectral curl of the half spectrum held in U: y fwd, z (fwd, curl, inv), y inv.  L may hold a box:
+// use_box where the result is used inside Omega only, use_tbox where the input is zero outside.
 template <typename T> cudaError_t curl_in_U(scfft_ctx* c, const Launch<T>& L, bool check_done) {
   cudaError_t e;
   if ((e = run(c, SCFFT_K_Y_FWD_U, [&] { return launch_y<T>(L, false, false, check_done); })) != cudaSuccess) return e;
@@ -613,7 +621,7 @@ scfft_status rhs_impl(scfft_ctx* c, double t, int left, const RhsIO& io, int* it
       CK(run(c, SCFFT_K_X_POWERLAW,
              [&] { return launch_x<T>(L, X_POWERLAW, pp, nullptr, nullptr, nullptr, 0, 0, false); }));
     }
-    CK(curl_in_U<T>(c, L, false));
+    CK(curl_in_U<T>(c, boxed(L), false));  // (used inside Omega only)
     CK(run(c, SCFFT_K_X_ASSEMBLE, [&] { return x_io<T>(L, X_ASSEMBLE, pp, io); }));
   }
   const int maxit = c->opt.max_iter;
@@ -1355,8 +1363,8 @@ bool capture_stage(scfft_ctx* c, cudaStream_t cs, cudaStream_t cs2, const PointP
                                  : launch_x<float>(L, X_POWERLAW, pp, nullptr, nullptr, nullptr, 0, 0, false);
     if (e != cudaSuccess) return false;
     if (launch_y<float>(L, false, false, false) != cudaSuccess) return false;
-    if (launch_z_curl<float>(L, false, 1.0 / (double)L.g.N) != cudaSuccess) return false;
-    if (launch_y<float>(L, false, true, false) != cudaSuccess) return false;
+    if (launch_z_curl<float>(boxed(L), false, 1.0 / (double)L.g.N) != cudaSuccess) return false;
+    if (launch_y<float>(boxed(L), false, true, false) != cudaSuccess) return false;
     if (launch_x_reg_io(L, X_ASSEMBLE, pp, nullptr, nullptr, nullptr, nullptr, warm32, 0, 0, false) != cudaSuccess)
       return false;
   }
@@ -1652,9 +1660,12 @@ scfft_status vjp_impl(scfft_ctx* c, const double* h, const double* lam, double* 
   PointParams pp = base_params(c);
   // forward j = C h (the power law's Jacobian needs it)
   CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_FWD_F64, pp, h, nullptr, nullptr, 0, 0, false); }));
-  CK(curl_in_U<T>(c, L, false));
+  // (read inside Omega only)
+  const Launch<T> LB = boxed(L), LT = tboxed(L);
+  CK(curl_in_U<T>(c, LB, false));
   CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_TO_F64, pp, nullptr, jf, nullptr, 0, 0, false); }));
-  // transposed iterations: lam_i = chi lam_{i+1} + C chi Phi (1 - chi) lam_{i+1}
+  // transposed iterations: lam_i = chi lam_{i+1} + C chi Phi (1 - chi) lam_{i+1}; Phi's result and the
+  // curl's input only in Omega's box (reverse mode 96^3 FP32, the lens: 944 -> 852 us)
   const double* cur = lam;
   for (int i = 0; i < K; ++i) {
     double* nxt = lb[i & 1];
@@ -1664,10 +1675,10 @@ scfft_status vjp_impl(scfft_ctx* c, const double* h, const double* lam, double* 
     }));
     CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_ADJ_PAD, pp, cur, nullptr, nullptr, 0, 0, false); }));
     CK(run(c, SCFFT_K_Y_FWD_P, [&] { return launch_y<T>(L, true, false, false); }));
-    CK(run(c, SCFFT_K_Z_KERNEL, [&] { return launch_z_kernel<T>(L, false); }));
-    CK(run(c, SCFFT_K_Y_INV_P, [&] { return launch_y<T>(L, true, true, false); }));
-    CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_ADJ_CROP, pp, nullptr, nullptr, nullptr, 0, 0, false); }));
-    CK(curl_in_U<T>(c, L, false));
+    CK(run(c, SCFFT_K_Z_KERNEL, [&] { return launch_z_kernel<T>(LT, false); }));
+    CK(run(c, SCFFT_K_Y_INV_P, [&] { return launch_y<T>(LT, true, true, false); }));
+    CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(LT, X_ADJ_CROP, pp, nullptr, nullptr, nullptr, 0, 0, false); }));
+    CK(curl_in_U<T>(c, LT, false));
     CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_ADJ_COMBINE, pp, cur, nxt, nullptr, 0, 0, false); }));
     cur = nxt;
   }
@@ -1678,8 +1689,8 @@ scfft_status vjp_impl(scfft_ctx* c, const double* h, const double* lam, double* 
       return cudaGetLastError();
     }));
   // u = -C e / mu0; e = E(j); j = C h
-  CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_ADJ_IN, pp, cur, nullptr, nullptr, 0, 0, false); }));
-  CK(curl_in_U<T>(c, L, false));
+  CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(LT, X_ADJ_IN, pp, cur, nullptr, nullptr, 0, 0, false); }));
+  CK(curl_in_U<T>(c, LT, false));
   CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_ADJ_POWERLAW, pp, jf, mu_jc, nullptr, 0, 0, false); }));
   CK(curl_in_U<T>(c, L, false));
   CK(run(c, SCFFT_K_OTHER, [&] { return launch_x<T>(L, X_TO_F64, pp, nullptr, mu_h, nullptr, 0, 0, false); }));

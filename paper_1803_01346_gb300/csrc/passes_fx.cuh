@@ -68,7 +68,7 @@ struct YArgs {
   const Ctrl* ctrl;
   int check_done;
   // planes z = zoff + blockIdx.y; rows outside [ylo, yhi): the forward pass reads them as zero, the
-  // unpadded inverse pass does not write them
+  // inverse pass does not write them
   int zoff, ylo, yhi;
 };
 
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
 #pragma unroll
       for (int k1 = 0; k1 < (PAD && INV ? R1 / 2 : R1); ++k1) {
         const int row = n1 + R2 * k1;
-        if (!INV || PAD || (row >= a.ylo && row < a.yhi)) col[(size_t)row * a.sx] = dbl_of(w[k1], U);
+        if (!INV || (row >= a.ylo && row < a.yhi)) col[(size_t)row * a.sx] = dbl_of(w[k1], U);
       }
     }
   }
@@ -156,7 +156,7 @@ struct ZArgs {
   int nx, ny, nz;
   const Ctrl* ctrl;
   int check_done;
-  int zlo, zhi;  // planes outside [zlo, zhi): the padded pass reads them as zero, the curl's does not write them
+  int ilo, ihi, olo, ohi;  // planes outside [ilo, ihi) read as zero, planes outside [olo, ohi) are not written
 };
 
 // |c| < 2^dexp(c)
@@ -170,11 +170,11 @@ __device__ __forceinline__ long long scaled62(double c, int e) {
 // One CTA takes TC columns (kx, y) of all three components: forward z transforms one after
 // another, the product on the points each thread itself finished (its "own slots" of the transpose
 // buffer, so the product needs no barrier), inverse transforms.  KIND 0: the smoothed curl on the
-// unpadded grid; KIND 1: the Biot-Savart kernel on the padded grid (half of the input planes are
+// unpadded grid (TB: of a field that is zero outside some planes); KIND 1: the Biot-Savart kernel on the padded grid (half of the input planes are
 // zero and half of the output planes are kept).  A 1-D grid: TC consecutive kx of one row per
 // CTA; the columns left over when HX is not a multiple of TC are packed TC (row, kx) pairs to a
 // CTA and run first.
-template <int R1, int R2, int TC, int KIND>
+template <int R1, int R2, int TC, int KIND, bool TB>
 __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
   constexpr int L = R1 * R2, NT = TC * R1;
   constexpr bool PR = KIND == 1;
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
 #pragma unroll
     for (int n2 = 0; n2 < NL; ++n2) {
       const int l = n1 + R1 * n2;
-      raw[n2] = (colok && (!PR || (l >= a.zlo && l < a.zhi))) ? ld_raw(col + q * cstride + l * zstride)
-                                                             : make_int4(0, 0, 0, 0);
+      raw[n2] = (colok && (!(PR || TB) || (l >= a.ilo && l < a.ihi))) ? ld_raw(col + q * cstride + l * zstride)
+                                                   : make_int4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int n2 = 0; n2 < NL; ++n2) m = top_of(m, raw[n2]);
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
 #pragma unroll
       for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) {
         const int l = n1 + R1 * m2;
-        if (PR || (l >= a.zlo && l < a.zhi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
+        if ((!PR && TB) || (l >= a.olo && l < a.ohi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
       }
     }
   }
@@ -378,7 +378,8 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
 // ---------------------------------------------------------------- x passes
 // As xwide_kernel (passes_wide.cuh), with the transforms in fixed point.  The rows between the
 // transforms are doubles in shared memory.
-template <int CIN, int COUT, int R1i, int R2i, int R2o>
+// SPLIT: each work item is one component of a tile (the passes that multiply by chi).
+template <int CIN, int COUT, int R1i, int R2i, int R2o, bool SPLIT>
 __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const int4* __restrict__ tw_in,
                                                    const int4* __restrict__ tw_out) {
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
@@ -403,7 +404,9 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
   fxc* Tp = Tb + p * TT;
   double part = 0.0;
   __syncthreads();
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int item = blockIdx.x; item < (SPLIT ? 3 * ntiles : ntiles); item += gridDim.x) {
+    const int tile = SPLIT ? item / 3 : item;
+    const int q0 = SPLIT ? item - 3 * tile : 0, q1 = SPLIT ? q0 + 1 : 3;
     const int gp = tile * P + p;
     const bool pok = gp < npairs;
     const int gq = pok ? gp : 0;
@@ -412,7 +415,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
     const size_t na0 = ((size_t)z * ny + ya) * XL;  // first node of the pair's first row
     if constexpr (CIN > 0) {
 #pragma unroll 1
-      for (int q = 0; q < 3; ++q) {
+      for (int q = q0; q < q1; ++q) {
         fxc v[R2i];
         int u = INT_MIN, want = INT_MIN;
         if (r < R1i) {
@@ -477,7 +480,15 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
           for (int q = 0; q < 3; ++q) RS[(q * P + p) * XL + x] = make_double2(va[q], vb[q]);
         }
       };
-      if (pok) {
+      if constexpr (SPLIT) {
+        if (pok) {
+          for (int x = r; x < XL; x += TP) {
+            double2* w = RS + (q0 * P + p) * XL + x;
+            if (!a.mask[na0 + x]) w->x = 0.0;
+            if (!a.mask[na0 + XL + x]) w->y = 0.0;
+          }
+        }
+      } else if (pok) {
 #pragma unroll 1
         for (int x = r; x < XL; x += TP) step(x);
       }
@@ -514,7 +525,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
     }
     if constexpr (COUT > 0) {
 #pragma unroll 1
-      for (int q = 0; q < 3; ++q) {
+      for (int q = q0; q < q1; ++q) {
         constexpr bool HALF = COUT == 2;
         constexpr int NL = HALF ? R2o / 2 : R2o;
         fxc v[R2o];
@@ -585,15 +596,17 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
 }
 
 // ---------------------------------------------------------------- launchers
-template <int CIN, int COUT, int R1i, int R2i, int R2o>
+template <int CIN, int COUT, int R1i, int R2i, int R2o, bool SPLIT = false>
 cudaError_t go_x(const Launch<double>& L, const XArgs<double>& a) {
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
-  constexpr auto k = xpass_kernel<CIN, COUT, R1i, R2i, R2o>;
+  if constexpr (S::MASKS && !SPLIT)
+    if (a.comp_split) return go_x<CIN, COUT, R1i, R2i, R2o, true>(L, a);
+  constexpr auto k = xpass_kernel<CIN, COUT, R1i, R2i, R2o, SPLIT>;
   const size_t smem = sizeof(fxc) * S::SM;
   allow_smem<k>();
   static const int resident = wide::resident_ctas(k, S::NT, smem);
   const int hp = (a.use_box ? a.by1 - a.by0 : a.g.ny) / 2;
-  const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P;
+  const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P * (SPLIT ? 3 : 1);
   const int grid = ntiles < resident ? ntiles : resident;
   const Work<double>& w = *L.w;
   launch_chained(k, dim3(grid), S::NT, smem, L.st, a, CIN == 2 ? w.fxp[0] : w.fxu[0], COUT == 2 ? w.fxp[0] : w.fxu[0]);

@@ -191,7 +191,7 @@ __global__ void zpass_reg2_kernel(float2* __restrict__ base, int rows, int sx, i
                                   const float* __restrict__ kt1, const float* __restrict__ kt2,
                                   const float* __restrict__ st0, const float* __restrict__ st1,
                                   const float* __restrict__ st2, float scale, const float4* __restrict__ kap4, int nx,
-                                  int ny, int nz, const Ctrl* ctrl, int check_done, int zlo, int zhi);
+                                  int ny, int nz, const Ctrl* ctrl, int check_done, int zlo, int zhi, int zin);
 
 template <int TC>
 __global__ void zpass_tm2_kernel(float2* __restrict__ base, int rows, int sx, int HX, int nzs,
@@ -210,8 +210,8 @@ cudaError_t go_y(const Launch<float>& L, float2* base, int rows, int sx, int HX,
   auto k = ypass_reg_kernel<float, R1, R2, TC, INV, PIN, POUT>;
   allow_smem<ypass_reg_kernel<float, R1, R2, TC, INV, PIN, POUT>>();
   // the padded forward pass and the curl's unpadded inverse pass of an Eq. 5 iteration: only
-  // the planes and rows of Omega's box
-  const bool box = L.use_box && (PIN || (INV && !POUT));
+  // the planes and rows of Omega's box; in the transposed iteration, the other two passes
+  const bool box = (L.use_box && (PIN || (INV && !POUT))) || (L.use_tbox && (POUT || (!INV && !PIN)));
   dim3 grid((HX + TC - 1) / TC, box ? L.bz1 - L.bz0 : L.g.nz, 3);
   static const int resident = [&] {  // CTAs resident at once: the prefetch distance
     if (!PF) return 0;
@@ -242,11 +242,12 @@ cudaError_t go_z(const Launch<float>& L, float2* base, int rows, int sx, int HX,
   const int nfull = HX / TC, rem = HX - nfull * TC;
   const dim3 grid = PACK ? dim3(nfull * rows + (rows * rem + TC - 1) / TC, 1, 1) : dim3((HX + TC - 1) / TC, rows, 1);
   const Work<float>& w = *L.w;
-  // box: the padded pass's input planes, or the curl pass's output planes (both Omega's box)
-  const bool box = L.use_box;
+  // box: the padded pass's input planes, or the curl pass's output planes (both Omega's box); tbox: the
+  // curl pass's input planes
+  const bool tbox = L.use_tbox && KIND == 0, box = L.use_box || tbox;
   launch_chained(k, dim3(grid), TC * R1, smem, L.st, base, rows, sx, HX, L.g.nz, tw, w.kt[0], w.kt[1], w.kt[2], w.st[0], w.st[1],
                                    w.st[2], (float)scale, w.kap4, L.g.nx, L.g.ny, L.g.nz, L.ctrl, chk ? 1 : 0,
-                                   box ? L.bz0 : 0, box ? L.bz1 : Lt);
+                                   box ? L.bz0 : 0, box ? L.bz1 : Lt, tbox ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -627,7 +628,8 @@ __global__ void __launch_bounds__(TC * R1, (R1 == R2 && KIND >= 1) ? 4 : 1) zpas
                                                              const float* __restrict__ st1,
                                                              const float* __restrict__ st2, float scale,
                                                              const float4* __restrict__ kap4, int nx, int ny, int nz,
-                                                             const Ctrl* ctrl, int check_done, int zlo, int zhi) {
+                                                             const Ctrl* ctrl, int check_done, int zlo, int zhi,
+                                                             int zin) {
   constexpr int L = R1 * R2;
   constexpr bool PR = (KIND >= 1);
   // KIND 2: the own-slot spectra of components 0 and 1 live in tensor memory instead of
@@ -708,8 +710,9 @@ __global__ void __launch_bounds__(TC * R1, (R1 == R2 && KIND >= 1) ? 4 : 1) zpas
   for (int q = 0; q < 3; ++q)
 #pragma unroll
     for (int n2 = 0; n2 < NL; ++n2)
-      // (input planes outside [zlo, zhi) are zero: the source vanishes outside Omega's box)
-      pre[q][n2] = (colok && (!PR || (n1 + R1 * n2 >= zlo && n1 + R1 * n2 < zhi)))
+      // (input planes outside [zlo, zhi) are zero: the source vanishes outside Omega's box; so does the
+      // curl's input in the transposed iteration, zin, where its output is kept on every plane)
+      pre[q][n2] = (colok && ((!PR && !zin) || (n1 + R1 * n2 >= zlo && n1 + R1 * n2 < zhi)))
                        ? col[q * cstride + (size_t)(n1 + R1 * n2) * zstride]
                        : make_float2(0.f, 0.f);
   if constexpr (OWN) {
@@ -870,7 +873,7 @@ __global__ void __launch_bounds__(TC * R1, (R1 == R2 && KIND >= 1) ? 4 : 1) zpas
           if (PR && m2 >= R2 / 2) continue;
           // (the curl's pass of an Eq. 5 iteration writes only the planes of Omega's box: the
           // masked curl downstream reads nothing else)
-          if (!PR && (n1 + R1 * m2 < zlo || n1 + R1 * m2 >= zhi)) continue;
+          if (!PR && !zin && (n1 + R1 * m2 < zlo || n1 + R1 * m2 >= zhi)) continue;
           col[q * cstride + (size_t)(n1 + R1 * m2) * zstride] = v[m2];
         }
       }
@@ -961,7 +964,7 @@ __global__ void __launch_bounds__(TC * R1, (R1 == R2 && KIND >= 1) ? 4 : 1) zpas
           if (PR && m2 >= R2 / 2) continue;
           // (the curl's pass of an Eq. 5 iteration writes only the planes of Omega's box: the
           // masked curl downstream reads nothing else)
-          if (!PR && (n1 + R1 * m2 < zlo || n1 + R1 * m2 >= zhi)) continue;
+          if (!PR && !zin && (n1 + R1 * m2 < zlo || n1 + R1 * m2 >= zhi)) continue;
           col[q * cstride + (size_t)(n1 + R1 * m2) * zstride] = v[m2];
         }
       }

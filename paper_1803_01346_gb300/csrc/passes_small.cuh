@@ -265,8 +265,8 @@ struct YArgs {
   const double2* tw;
   const Ctrl* ctrl;
   int check_done;
-  // planes from zoff; rows outside [ylo, yhi): the forward pass reads them as zero, the unpadded
-  // inverse pass does not write them
+  // planes from zoff; rows outside [ylo, yhi): the forward pass reads them as zero, the inverse
+  // pass need not write them
   int zoff, ylo, yhi;
 };
 // 16 and 32 points: one warp a CTA, two or one columns (component, plane, kx).
@@ -286,7 +286,7 @@ template <int L, bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass
   if (done) return;
   Lanes<L>::template run<INV, SH>(&v, row, &tw);
   const int o = Lanes<L>::out(row);
-  if (ok && (!INV || (PAD ? o < L / 2 : o >= a.ylo && o < a.yhi))) col[(size_t)o * a.sx] = v;
+  if (ok && (!INV || (o >= a.ylo && o < a.yhi && (!PAD || o < L / 2)))) col[(size_t)o * a.sx] = v;
 }
 // 64 points: 32-thread CTAs, 8 threads a column and 8 points a thread.
 template <bool INV, bool PAD> __global__ void __launch_bounds__(32) ypass64_kernel(const YArgs a) {
@@ -330,7 +330,7 @@ struct ZArgs {
   int nx, ny, nz;
   const Ctrl* ctrl;
   int check_done;
-  int zlo, zhi;  // planes outside [zlo, zhi): the padded pass reads them as zero, the curl's does not write them
+  int ilo, ihi, olo, ohi;  // planes outside [ilo, ihi) read as zero, planes outside [olo, ohi) are not written
 };
 // 16 and 32 points: one CTA of three warps, a component to a warp, for two or one columns (kx, y);
 // the three spectra meet in shared memory, where each thread takes the product of its own component.
@@ -348,7 +348,7 @@ template <int L, int KIND> __global__ void __launch_bounds__(96) zpass_lanes_ker
   const size_t zstride = (size_t)a.rows * a.sx;
   double2* col = a.base + (size_t)q * a.nzs * zstride + (size_t)y * a.sx + kx;
   double2 v = mk(0.0, 0.0), tw = mk(0.0, 0.0);
-  if (!(PR && l >= L / 2) && ok && (!PR || (l >= a.zlo && l < a.zhi))) v = col[l * zstride];
+  if (!(PR && l >= L / 2) && ok && l >= a.ilo && l < a.ihi) v = col[l * zstride];
   if (L > 16) tw = a.tw[Lanes<L>::twiddle(l)];
   // the factors of the product i s (k x F): the two that this component takes
   const int qb = q == 2 ? 0 : q + 1, qc = q == 0 ? 2 : q - 1;
@@ -375,7 +375,7 @@ template <int L, int KIND> __global__ void __launch_bounds__(96) zpass_lanes_ker
   const double2 x = mk(kb * Fc.x - kc * Fb.x, kb * Fc.y - kc * Fb.y);
   v = PR ? mk(-x.y, x.x) : mk(-s * x.y, s * x.x);
   Lanes<L>::template run<true, SH>(&v, l, &tw);
-  if (ok && (PR ? o < L / 2 : o >= a.zlo && o < a.zhi)) col[o * zstride] = v;
+  if (ok && o >= a.olo && o < a.ohi && (!PR || o < L / 2)) col[o * zstride] = v;
 }
 // 64 points (always the padded pass): four columns (kx, y) a CTA, its threads over (component,
 // residue, column), 8 points a thread; the product over the spectra in shared memory.
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(96) zpass64_kernel(const ZArgs a) {
 #pragma unroll
   for (int n2 = 0; n2 < 8; ++n2) {
     const int l = n1 + 8 * n2;
-    v[n2] = (n2 < 4 && ok && l >= a.zlo && l < a.zhi) ? col[l * zstride] : mk(0.0, 0.0);
+    v[n2] = (n2 < 4 && ok && l >= a.ilo && l < a.ihi) ? col[l * zstride] : mk(0.0, 0.0);
   }
   for (int i = t; i < L; i += NT) tw[i] = a.tw[i];
   __syncthreads();

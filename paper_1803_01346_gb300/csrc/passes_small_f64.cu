@@ -45,8 +45,8 @@ cudaError_t launch_y(const Launch<double>& L, bool padded, bool inverse, bool ch
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
   // the padded forward pass and the curl's unpadded inverse pass of an Eq. 5 iteration: only the
-  // planes and rows of Omega's box
-  const bool box = L.use_box && padded != inverse;
+  // planes and rows of Omega's box; in the transposed iteration, the other two passes
+  const bool box = padded != inverse ? L.use_box : L.use_tbox;
   a.zoff = box ? L.bz0 : 0;
   a.ylo = box ? L.by0 : 0;
   a.yhi = box ? L.by1 : a.rows;
@@ -87,8 +87,12 @@ cudaError_t launch_z(const Launch<double>& L, bool padded, bool check_done, doub
   a.nx = g.nx; a.ny = g.ny; a.nz = g.nz;
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
-  a.zlo = L.use_box ? L.bz0 : 0;  // the source box of an Eq. 5 iteration
-  a.zhi = L.use_box ? L.bz1 : Lz;
+  // Omega's box: the padded pass's input and the curl's output, or, transposed, the other two
+  const bool in = padded ? L.use_box : L.use_tbox, out = padded ? L.use_tbox : L.use_box;
+  a.ilo = in ? L.bz0 : 0;
+  a.ihi = in ? L.bz1 : Lz;
+  a.olo = out ? L.bz0 : 0;
+  a.ohi = out ? L.bz1 : Lz;
   if (!padded) {
     if (Lz == 16) return go_z<16, 0>(a, L.st);
     if (Lz == 32) return go_z<32, 0>(a, L.st);

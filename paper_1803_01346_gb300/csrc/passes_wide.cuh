@@ -92,9 +92,13 @@ struct XArgs {
   Ctrl* ctrl;
   double* partials;
   int check_done;
-  // mask/pad pass of an Eq. 5 iteration: only the rows of Omega's box (y in [by0, by1), z in
-  // [bz0, bz1)); the source vanishes outside, and nothing downstream reads the rows left out
+  // mask/pad pass of an Eq. 5 iteration, and the passes of the transposed one that multiply by chi:
+  // only the rows of Omega's box (y in [by0, by1), z in [bz0, bz1)); the source vanishes outside,
+  // and nothing downstream reads the rows left out
   int use_box, by0, by1, bz0, bz1;
+  // those passes: each work item is one component of a tile.  The box holds few tiles (64 x 64 x 96 shield: 293
+  // of four row pairs, two CTAs of 64 threads an SM): FP64 mask/pad 47 -> 25 us there
+  int comp_split;
 };
 
 // What the update pass takes from the device, so that a captured launch serves every iteration:
@@ -281,10 +285,14 @@ template <int CIN, int COUT, int R1i, int R2i, int R2o> struct WX {
   static constexpr int KX = CIN == 2 ? R1i / 2 : R1i;
   static constexpr int TT = wide::cmax(CIN ? R2i * (R1i + 1) : 1, COUT ? R2o * (R1o + 1) : 1);
   static constexpr int TWI = CIN ? Li : 0, TWO = COUT ? Lo : 0;
+  // whether the node-wise step may be the product by chi (mask/pad, its transposed counterpart), which
+  // leaves the components independent
+  static constexpr bool MASKS = (CIN == 1 && COUT == 2) || (CIN == 2 && COUT == 1);
   static constexpr int SM = TWI + TWO + 3 * P * XL + P * TT;  // complex values of shared memory
 };
 
-template <typename T, int CIN, int COUT, int R1i, int R2i, int R2o>
+// SPLIT: each work item is one component of a tile (the passes that multiply by chi).
+template <typename T, int CIN, int COUT, int R1i, int R2i, int R2o, bool SPLIT>
 __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
   typedef typename cplx_of<T>::type V;
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
@@ -309,7 +317,9 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
   V* Tp = Tb + p * TT;
   double part = 0.0;
   __syncthreads();
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int item = blockIdx.x; item < (SPLIT ? 3 * ntiles : ntiles); item += gridDim.x) {
+    const int tile = SPLIT ? item / 3 : item;
+    const int q0 = SPLIT ? item - 3 * tile : 0, q1 = SPLIT ? q0 + 1 : 3;
     const int gp = tile * P + p;
     const bool pok = gp < npairs;
     const int gq = pok ? gp : 0;
@@ -318,7 +328,7 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
     const size_t na0 = ((size_t)z * ny + ya) * XL;  // first node of the pair's first row
     if constexpr (CIN > 0) {
 #pragma unroll 1
-      for (int q = 0; q < 3; ++q) {
+      for (int q = q0; q < q1; ++q) {
         if (r < R1i) {
           const V* ra = a.spec_in + ((size_t)(q * nz + z) * a.in_rows + ya) * a.in_sx;
           const V* rb = ra + a.in_sx;
@@ -351,18 +361,28 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
         __syncwarp();
       }
       // the node-wise step on the nodes x = r + TP j of both rows of the lane's pair
+      if constexpr (SPLIT) {
+        if (pok) {
+          for (int x = r; x < XL; x += TP) {
+            V* w = RS + (q0 * P + p) * XL + x;
+            if (!a.mask[na0 + x]) w->x = 0;
+            if (!a.mask[na0 + XL + x]) w->y = 0;
+          }
+        }
+      } else {
 #pragma unroll 1
-      for (int x = r; x < XL; x += TP) {
-        if (!pok) continue;
-        V u[3];
+        for (int x = r; x < XL; x += TP) {
+          if (!pok) continue;
+          V u[3];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) u[q] = RS[(q * P + p) * XL + x];
-        T va[3] = {u[0].x, u[1].x, u[2].x}, vb[3] = {u[0].y, u[1].y, u[2].y};
-        part += node_step<T>(a, up, na0 + x, va);
-        part += node_step<T>(a, up, na0 + XL + x, vb);
-        if (COUT > 0) {
+          for (int q = 0; q < 3; ++q) u[q] = RS[(q * P + p) * XL + x];
+          T va[3] = {u[0].x, u[1].x, u[2].x}, vb[3] = {u[0].y, u[1].y, u[2].y};
+          part += node_step<T>(a, up, na0 + x, va);
+          part += node_step<T>(a, up, na0 + XL + x, vb);
+          if (COUT > 0) {
 #pragma unroll
-          for (int q = 0; q < 3; ++q) RS[(q * P + p) * XL + x] = mk(va[q], vb[q]);
+            for (int q = 0; q < 3; ++q) RS[(q * P + p) * XL + x] = mk(va[q], vb[q]);
+          }
         }
       }
       __syncwarp();
@@ -397,7 +417,7 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
     }
     if constexpr (COUT > 0) {
 #pragma unroll 1
-      for (int q = 0; q < 3; ++q) {
+      for (int q = q0; q < q1; ++q) {
         if (r < R1o) {
           V u[R2o];
 #pragma unroll
@@ -449,15 +469,17 @@ __global__ void __launch_bounds__(64) xwide_kernel(const XArgs<T> a) {
 // ---------------------------------------------------------------- launchers
 namespace wide {
 
-template <typename T, int CIN, int COUT, int R1i, int R2i, int R2o>
+template <typename T, int CIN, int COUT, int R1i, int R2i, int R2o, bool SPLIT = false>
 cudaError_t go_x(const XArgs<T>& a, cudaStream_t st) {
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
-  constexpr auto k = xwide_kernel<T, CIN, COUT, R1i, R2i, R2o>;
+  if constexpr (S::MASKS && !SPLIT)
+    if (a.comp_split) return go_x<T, CIN, COUT, R1i, R2i, R2o, true>(a, st);
+  constexpr auto k = xwide_kernel<T, CIN, COUT, R1i, R2i, R2o, SPLIT>;
   const size_t smem = sizeof(typename cplx_of<T>::type) * S::SM;
   allow_smem<k>();
   static const int resident = resident_ctas(k, S::NT, smem);
   const int hp = (a.use_box ? a.by1 - a.by0 : a.g.ny) / 2;
-  const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P;
+  const int ntiles = ((a.use_box ? a.bz1 - a.bz0 : a.g.nz) * hp + S::P - 1) / S::P * (SPLIT ? 3 : 1);
   const int grid = ntiles < resident ? ntiles : resident;
   launch_chained(k, dim3(grid), S::NT, smem, st, a);
   return checked_launch("xwide_kernel", dim3(grid), S::NT, smem);
@@ -541,7 +563,8 @@ static cudaError_t launch_x_impl(const Launch<T>& L, XMode mode, const PointPara
   a.ctrl = L.ctrl;
   a.partials = L.partials;
   a.check_done = check_done ? 1 : 0;
-  a.use_box = (L.use_box && mode == X_MASKPAD) ? 1 : 0;
+  a.use_box = (L.use_box && mode == X_MASKPAD) || (L.use_tbox && (mode == X_ADJ_CROP || mode == X_ADJ_IN));
+  a.comp_split = a.use_box && (mode == X_MASKPAD || mode == X_ADJ_CROP);
   a.by0 = L.by0;
   a.by1 = L.by1;
   a.bz0 = L.bz0;

@@ -14,11 +14,11 @@ template <int R1, int R2, bool INV, bool PAD> cudaError_t go_y(const Launch<doub
   launch_chained(k, dim3(grid), TC * R1, smem, L.st, a);
   return checked_launch("fx ypass_kernel", grid, TC * R1, smem);
 }
-template <int R1, int R2, int KIND> cudaError_t go_z(const Launch<double>& L, const ZArgs& a) {
+template <int R1, int R2, int KIND, bool TB = false> cudaError_t go_z(const Launch<double>& L, const ZArgs& a) {
   constexpr int TC = R1 >= 8 ? 4 : 8;
   constexpr int PADZ = TC < 8 ? TC : 0;
   constexpr int CS = cmax(R2 * (R1 * TC + PADZ), R1 * (R2 * TC + PADZ));
-  constexpr auto k = zpass_kernel<R1, R2, TC, KIND>;
+  constexpr auto k = zpass_kernel<R1, R2, TC, KIND, TB>;
   const size_t smem = sizeof(fxc) * (R1 * R2 + 3 * CS);
   allow_smem<k>();
   const int nfull = a.HX / TC, rem = a.HX - nfull * TC;
@@ -39,8 +39,8 @@ cudaError_t launch_y(const Launch<double>& L, bool padded, bool inverse, bool ch
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
   // the padded forward pass and the curl's unpadded inverse pass of an Eq. 5 iteration: only the
-  // planes and rows of Omega's box
-  const bool box = L.use_box && padded != inverse;
+  // planes and rows of Omega's box; in the transposed iteration, the other two passes
+  const bool box = padded != inverse ? L.use_box : L.use_tbox;
   a.zoff = box ? L.bz0 : 0;
   a.ylo = box ? L.by0 : 0;
   a.yhi = box ? L.by1 : a.rows;
@@ -80,9 +80,13 @@ cudaError_t launch_z(const Launch<double>& L, bool padded, bool check_done, doub
   a.nx = g.nx; a.ny = g.ny; a.nz = g.nz;
   a.ctrl = L.ctrl;
   a.check_done = check_done ? 1 : 0;
-  a.zlo = L.use_box ? L.bz0 : 0;  // the source box of an Eq. 5 iteration
-  a.zhi = L.use_box ? L.bz1 : Lz;
-#define ZCASE_U(LL, R1, R2) case LL: return go_z<R1, R2, 0>(L, a);
+  // Omega's box: the padded pass's input and the curl's output, or, transposed, the other two
+  const bool in = padded ? L.use_box : L.use_tbox, out = padded ? L.use_tbox : L.use_box;
+  a.ilo = in ? L.bz0 : 0;
+  a.ihi = in ? L.bz1 : Lz;
+  a.olo = out ? L.bz0 : 0;
+  a.ohi = out ? L.bz1 : Lz;
+#define ZCASE_U(LL, R1, R2) case LL: return L.use_tbox ? go_z<R1, R2, 0, true>(L, a) : go_z<R1, R2, 0>(L, a);
 #define ZCASE_P(LL, R1, R2) case LL: return go_z<R1, R2, 1>(L, a);
   if (padded) {
     switch (Lz) { WIDE_PADDED(ZCASE_P) }

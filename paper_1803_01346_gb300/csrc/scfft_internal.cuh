@@ -163,6 +163,9 @@ struct Launch {
   // padded z pass's input) skip everything outside the box, where it is zero.
   int by0 = 0, by1 = 0, bz0 = 0, bz1 = 0;
   bool use_box = false;
+  // The transposed iteration of the reverse mode: Phi's result is used, and the curl's input nonzero, in the
+  // same box only.  (At most one of the two is set.)
+  bool use_tbox = false;
 };
 
 // Programmatic dependent launch.  The passes of one transform or iteration follow each other on one

@@ -170,7 +170,8 @@ cudaError_t go_y_tma(const Launch<float>& L, const CUtensorMap& map, float2* bas
   typedef YT<R1, R2, TC, PIN> S;
   auto k = ypass_tma_kernel<R1, R2, TC, INV, PIN, POUT>;
   allow_smem<ypass_tma_kernel<R1, R2, TC, INV, PIN, POUT>>();
-  const bool box = L.use_box && PIN;  // the forward pass of an Eq. 5 iteration: Omega's box only
+  // the forward pass of an Eq. 5 iteration, the inverse pass of the transposed one: Omega's box only
+  const bool box = (L.use_box && PIN) || (L.use_tbox && POUT);
   const int nzp = box ? L.bz1 - L.bz0 : L.g.nz;
   const int ntiles = ((HX + TC - 1) / TC) * 3 * nzp;
   static const int resident = [&] {  // one wave of resident CTAs (the kernel loops over tiles)
@@ -184,7 +185,7 @@ cudaError_t go_y_tma(const Launch<float>& L, const CUtensorMap& map, float2* bas
   const int inject = (L.fault && *L.fault == SCFFT_FAULT_TMA_WAIT) ? 1 : 0;
   if (inject) *L.fault = 0;  // one shot
   launch_chained(k, dim3(grid), TC * R1, S::smem, L.st, map, base, rows, sx, HX, L.g.nz, tw, L.ctrl, chk ? 1 : 0, inject,
-                                      box ? L.bz0 : 0, nzp, box ? L.by0 : 0, box ? L.by1 : rows);
+                                      box ? L.bz0 : 0, nzp, box && PIN ? L.by0 : 0, box && PIN ? L.by1 : rows);
   return cudaGetLastError();
 }
 

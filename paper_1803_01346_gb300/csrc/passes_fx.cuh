@@ -2,13 +2,16 @@
 // and fields are doubles in memory, transforms and spectral products run on 64-bit integers, the
 // node-wise steps in FP64.
 //
-// What bounds them is instruction issue on the integer pipes (additions 2, twiddles about 20
-// instructions a point), not the FP64 pipe, which kept the FP64 passes before these 76% busy.
-// Measured on 64 x 64 x 96 with a shield's box, FP64 | double-float passes before | these: padded z
-// 589 | 306 | 134 us, Eq. 5 update 177 | 122 | 64, padded y inverse 127 | 71 | 32, curl z 79 | 51 | 33;
-// one right-hand side 10.4 | 6.2 | 3.3 ms.  A length L = R1 R2 transform is two register stages with
-// one shared-memory transpose; every length is compiled on its own; the component loops stay
-// rolled, so that a kernel's four unrolled DFT bodies stay within the instruction cache.
+// What bounds them is latency and issue on the integer pipes (additions 2, twiddles about 20
+// instructions a point): the padded z pass runs 10 warps an SM, by shared memory and registers, at 41%
+// issue, the y passes 16 to 20 warps at 55 to 60%; not the FP64 pipe, which kept the FP64 passes
+// before these 76% busy.  Measured on 64 x 64 x 96 with a shield's box, us a launch, FP64 |
+// double-float passes before | these: padded z 589 | 306 | 141, Eq. 5 update 177 | 122 | 65, padded y
+// inverse 127 | 71 | 33, curl z 79 | 51 | 33; one right-hand side 10.4 | 6.2 | 2.9 ms.  A length L = R1 R2
+// transform is two register stages with one shared-memory transpose; every length is compiled on its
+// own; the component loops stay rolled, so that a kernel's four unrolled DFT bodies stay within the
+// instruction cache.  (Reading a component's input during the transform before it, in the z pass: 141 us
+// either way.)
 #pragma once
 #include <limits.h>
 
@@ -170,8 +173,10 @@ __device__ __forceinline__ long long scaled62(double c, int e) {
 // One CTA takes TC columns (kx, y) of all three components: forward z transforms one after
 // another, the product on the points each thread itself finished (its "own slots" of the transpose
 // buffer, so the product needs no barrier), inverse transforms.  KIND 0: the smoothed curl on the
-// unpadded grid (TB: of a field that is zero outside some planes); KIND 1: the Biot-Savart kernel on the padded grid (half of the input planes are
-// zero and half of the output planes are kept).  A 1-D grid: TC consecutive kx of one row per
+// unpadded grid; KIND 1: the Biot-Savart kernel on the padded grid (half of the input planes are
+// zero and half of the output planes are kept).  Omega's box: KIND 1 reads and KIND 0 writes its
+// planes only; TB, the transposed iteration's form, the other way round (run-time ranges on both
+// sides of both cost Phi 96^3 557 us against 552).  A 1-D grid: TC consecutive kx of one row per
 // CTA; the columns left over when HX is not a multiple of TC are packed TC (row, kx) pairs to a
 // CTA and run first.
 template <int R1, int R2, int TC, int KIND, bool TB>
@@ -369,7 +374,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
 #pragma unroll
       for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) {
         const int l = n1 + R1 * m2;
-        if ((!PR && TB) || (l >= a.olo && l < a.ohi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
+        if (PR != TB || (l >= a.olo && l < a.ohi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
       }
     }
   }

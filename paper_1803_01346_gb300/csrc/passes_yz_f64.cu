@@ -87,7 +87,7 @@ cudaError_t launch_z(const Launch<double>& L, bool padded, bool check_done, doub
   a.olo = out ? L.bz0 : 0;
   a.ohi = out ? L.bz1 : Lz;
 #define ZCASE_U(LL, R1, R2) case LL: return L.use_tbox ? go_z<R1, R2, 0, true>(L, a) : go_z<R1, R2, 0>(L, a);
-#define ZCASE_P(LL, R1, R2) case LL: return go_z<R1, R2, 1>(L, a);
+#define ZCASE_P(LL, R1, R2) case LL: return L.use_tbox ? go_z<R1, R2, 1, true>(L, a) : go_z<R1, R2, 1>(L, a);
   if (padded) {
     switch (Lz) { WIDE_PADDED(ZCASE_P) }
   } else {

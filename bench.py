@@ -613,7 +613,7 @@ def bench_ours(args, ws, rank, local):
     fp64_value = N * (ctx64.stats()["rhs_calls"] - c0) / (e4.elapsed_time(e5) * 1e-3)
     fp64_ms_per_step = e4.elapsed_time(e5) / k64
     del ctx64
-    # the double-float path (FP64-equivalent transforms on the FP32 pipes) over the same steps
+    # the FP64-equivalent mode (SCFFT_PREC_DF64, the FP64 passes) over the same steps
     cdf = make_ctx(S, cfg, S.PREC_DF64)
     stdf = [state[0], state[1], h.clone(), warm.clone()]
     torch.cuda.synchronize()
@@ -629,7 +629,7 @@ def bench_ours(args, ws, rank, local):
             "speedup_vs_fp64": fp64_ms_per_step / (e10.elapsed_time(e11) / k64),
             "iters_per_rhs": (d1["iterations"] - d0["iterations"]) / max(1, d1["rhs_calls"] - d0["rhs_calls"]),
             "error_vs_fp64": df64_err,
-            "what": "SCFFT_PREC_DF64: double-float FFT passes (hi + lo FP32), node-wise law and stages in FP64"}
+            "what": "SCFFT_PREC_DF64: the FP64 passes (64-bit block fixed-point transforms), node-wise law and stages in FP64"}
     del cdf, stdf
 
     # the local-stencil curl option: its own trajectory from the virgin state (a state of the

@@ -44,14 +44,18 @@ template <int R> __device__ __forceinline__ int want_unit(int u, int m) {
   const int w = u + fx_bits(m) - fx_head(R);
   return w > u ? w : u;
 }
-// Largest p over the threads of a column (same t % TC) into *slot[c].
-template <int TC> __device__ __forceinline__ void column_max(int* slot, int p) {
+// Largest p over the threads of a column (same t % TC) into slot[c], for a CTA of NT threads.  With 48
+// threads the second warp has 16 lanes, and a shuffle must not read the others: the butterfly stays within
+// groups of W lanes, which exist whole in every warp, and atomicMax joins the groups.
+template <int TC, int NT> __device__ __forceinline__ void column_max(int* slot, int p) {
+  constexpr int W = NT % 32 ? NT % 32 : 32;
+  static_assert((W & (W - 1)) == 0 && W >= TC && W % TC == 0, "a CTA ends in a power of two of lanes, whole columns");
 #pragma unroll
-  for (int o = TC; o < 32; o <<= 1) {
+  for (int o = TC; o < W; o <<= 1) {
     const int q = __shfl_xor_sync(0xffffffffu, p, o);
     p = q > p ? q : p;
   }
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (W - 1);
   if (lane < TC) atomicMax(slot + lane, p);
 }
 // v, in unit u, to unit U >= u
@@ -120,7 +124,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
     v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<INV>(v[k2], tw[n1 * k2]);
     m = fx_or(fx_or(m, v[k2].x), v[k2].y);
   }
-  column_max<TC>(unit, want_unit<R1>(u, m));
+  column_max<TC, NT>(unit, want_unit<R1>(u, m));
   __syncthreads();
   const int U = unit[c];
   to_unit<R2>(v, u, U);
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<false>(v[k2], tw[n1 * k2]);
       m = fx_or(fx_or(m, v[k2].x), v[k2].y);
     }
-    column_max<TC>(unit[q], want_unit<R1>(u, m));
+    column_max<TC, NT>(unit[q], want_unit<R1>(u, m));
     __syncthreads();
     to_unit<R2>(v, u, unit[q][c]);
 #pragma unroll
@@ -357,7 +361,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       }
       p = want_unit<R2>(u, m);
     }
-    column_max<TC>(unit[3 + q], p);
+    column_max<TC, NT>(unit[3 + q], p);
     __syncthreads();  // units known, every own slot of this buffer read
     const int U = unit[3 + q][c];
     if (n1 < R2) {

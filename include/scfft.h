@@ -51,8 +51,9 @@ typedef enum {
  * are FP64 in every mode.
  *   SCFFT_PREC_F64   FP64 spectra and fields, FP64 stage sums.  The transforms run on 64-bit
  *                    integers with an exponent per block of values (nearer to exact arithmetic
- *                    than FP64 transforms), or, with every axis at most 32, in FP64.  Values below
- *                    2.2e-308 count as zero; an infinity or a NaN makes the pencils it meets NaN.
+ *                    than FP64 transforms), or, with every axis at most 32, in FP64.  Either way
+ *                    over the whole range of FP64; an infinity or a NaN makes the pencils it
+ *                    meets NaN.
  *   SCFFT_PREC_F32   FP32 transforms and stages, FP64 state with compensated sums.
  *   SCFFT_PREC_DF64  the same as SCFFT_PREC_F64 (kept for programs that ask for it: a faster
  *                    FP64-equivalent form, which the FP64 passes have become). */

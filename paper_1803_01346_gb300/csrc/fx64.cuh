@@ -15,8 +15,8 @@
 // Rounding therefore happens at 2^-57 or so of the largest value of a block instead of at 2^-53 of
 // each value, and additions are exact: against exact arithmetic the transform of 16 to 256 points
 // comes out 2 to 4 times nearer than the FP64 one (what is left is the rounding of the results to
-// doubles).  A block that holds an infinity or a NaN gives NaN (unit kNanUnit); doubles below
-// 2.2e-308 read as zero.
+// doubles).  A block that holds an infinity or a NaN gives NaN (unit kNanUnit).
+// Subnormal doubles are read and written (a unit below that of the smallest normal is as good as any).
 //
 // Unit exponents are kept in the bias of FP64: value = v 2^(u - 1075).
 #pragma once
@@ -164,27 +164,34 @@ FXHD int fx_top(int m, int hi) {
   const int a = hi & 0x7fffffff;
   return a > m ? a : m;
 }
-FXHD int fx_exp_of(int m) { return (m >> 20) > 64 ? (m >> 20) : 64; }
+FXHD int fx_exp_of(int m) { return (m >> 20) > 1 ? (m >> 20) : 1; }
 FXHD int fx_unit_of(int et, int head) { return et >= 0x7ff ? kNanUnit : et - (head - 53); }
-// the double (hi, lo) in the unit fx_unit_of(et, HEAD), cut toward zero
+// the double (hi, lo) in the unit fx_unit_of(et, HEAD), cut toward zero.  Zeros and subnormals have
+// the exponent 1 and no leading bit.
 template <int HEAD> FXHD long long fx_from_double(int hi, unsigned lo, int et) {
-  int d = et - ((hi >> 20) & 0x7ff);
-  d = d < 63 ? d : 63;
-  unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const int a = hi & 0x7fffffff, e = fx_exp_of(a);
+  const int d = et - e < 63 ? et - e : 63;
+  unsigned long long m = ((unsigned long long)(unsigned)(a - ((e - 1) << 20)) << 32) | lo;
   m = (m << (HEAD - 53)) >> d;
   return hi < 0 ? -(long long)m : (long long)m;
 }
-// v 2^(u - 1075) as a double, rounded to nearest (ties away from zero); NaN from kNanUnit / 2 on
-FXHD unsigned long long fx_to_bits(long long v, int u) {
+// v 2^(u - 1075) as a double, rounded to nearest (ties away from zero); NaN from kNanUnit / 2 on.
+// PLAIN: for a unit in which every value but 0 is a normal double (fx_plain).
+FXHD bool fx_plain(int u) { return (unsigned)(u - 53) <= 2036u - 53u; }
+template <bool PLAIN> FXHD unsigned long long fx_to_bits(long long v, int u) {
   const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
   const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
   const int z = ah ? fx_clz(ah) : 32 + fx_clz(al);  // 1 .. 64
   const int e = u + 11 - z;
-  unsigned long long m = ((a << (z - 1)) + 0x200) >> 10;
+  const unsigned long long n = a << (z - 1);
+  unsigned long long m = (n + 0x200) >> 10;
   m += (unsigned long long)(unsigned)(e - 1) << 52;
   if (a == 0) m = 0;
-  else if ((unsigned)(e - 1) >= 2046u) m = e <= 0 ? 0 : 0x7ff0000000000000ull;
-  if (u >= kNanUnit / 2) return 0x7ff8000000000000ull;
+  if (!PLAIN) {
+    if (a != 0 && e <= 0) m = e > -53 ? (n + (1ull << (10 - e))) >> (11 - e) : 0;  // subnormal
+    if (a != 0 && e > 2046) m = 0x7ff0000000000000ull;
+    if (u >= kNanUnit / 2) return 0x7ff8000000000000ull;
+  }
   return m | ((unsigned long long)v & 0x8000000000000000ull);
 }
 // bits a block's values may use, from the OR of their high words' magnitudes (fx_or)

@@ -32,9 +32,32 @@ __device__ __forceinline__ int top_of(int m, int4 r) { return fx_top(fx_top(m, r
 template <int HEAD> __device__ __forceinline__ fxc fx_of(int4 r, int et) {
   return mk(fx_from_double<HEAD>(r.y, (unsigned)r.x, et), fx_from_double<HEAD>(r.w, (unsigned)r.z, et));
 }
-__device__ __forceinline__ double2 dbl_of(fxc v, int u) {
-  return make_double2(__longlong_as_double((long long)fx_to_bits(v.x, u)),
-                      __longlong_as_double((long long)fx_to_bits(v.y, u)));
+template <bool PLAIN> __device__ __forceinline__ double2 dbl_of(fxc v, int u) {
+  return make_double2(__longlong_as_double((long long)fx_to_bits<PLAIN>(v.x, u)),
+                      __longlong_as_double((long long)fx_to_bits<PLAIN>(v.y, u)));
+}
+// A thread's block of doubles (R points, those from N on zero) in fixed point; m: its fx_top, made 0 for
+// a block of zeros alone and 1 for one that lies below 2^-1042.  Returns the block's exponent.
+template <int R, int N> __device__ __forceinline__ int block_in(fxc* v, const int4* raw, int& m) {
+  if (m == 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) m |= raw[i].x | raw[i].z;
+    m = m != 0;
+  }
+  const int et = fx_exp_of(m);
+#pragma unroll
+  for (int i = 0; i < R; ++i) v[i] = i < N ? fx_of<fx_head(R)>(raw[i < N ? i : 0], et) : mk(0ll, 0ll);
+  return et;
+}
+// The unit of a block of zeros, which has no part in the choice of a pencil's unit.
+constexpr int kNoUnit = -(1 << 20);
+// Writing results: whether the unit is plain (fx_plain; zeros alone are) is asked once a block and f called
+// with std::true_type or std::false_type: with the checks at every value a 64 x 64 x 96 right-hand side took
+// 3.02 ms, without 2.79, and Phi at 96^3 569 us, without 500.
+__device__ __forceinline__ bool plain_unit(int u) { return fx_plain(u) || u < kNoUnit / 2; }
+template <typename F> __device__ __forceinline__ void by_unit(bool plain, F&& f) {
+  if (__builtin_expect(plain, 1)) f(std::true_type{});
+  else f(std::false_type{});
 }
 __device__ __forceinline__ fxc shfl_fx(fxc v, int s) {
   return mk(__shfl_sync(0xffffffffu, v.x, s), __shfl_sync(0xffffffffu, v.y, s));
@@ -81,9 +104,10 @@ struct YArgs {
 
 // grid (ceil(HX / TC), planes, 3), TC columns of one (component, plane) per CTA.  PAD: the
 // zero-padded transform (forward: only the first half of the rows is read; inverse: only the
-// first half is kept).
+// first half is kept).  192 points (R2 = 12) are held to ten CTAs an SM: left alone the compiler takes registers
+// for nine (forward y on the lens's box at 96 x 96 x 64: 25.4 us against 18.4).
 template <int R1, int R2, int TC, bool INV, bool PAD>
-__global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
+__global__ void __launch_bounds__(TC * R1, R2 == 12 ? 10 : 0) ypass_kernel(const YArgs a) {
   constexpr int L = R1 * R2, NT = TC * R1;
   constexpr int S2 = R1 * TC + (TC < 8 ? TC : 0);  // 8 lanes of a 16-byte access on distinct banks
   constexpr bool HALF = PAD && !INV;
@@ -108,13 +132,12 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
                                                                : make_int4(0, 0, 0, 0);
   }
   for (int i = t; i < L; i += NT) tw[i] = a.tw[i];
-  if (t < TC) unit[t] = INT_MIN;
+  if (t < TC) unit[t] = kNoUnit;
 #pragma unroll
   for (int n2 = 0; n2 < NL; ++n2) m = top_of(m, raw[n2]);
-  const int et = fx_exp_of(m);
   fxc v[R2];
-#pragma unroll
-  for (int n2 = 0; n2 < R2; ++n2) v[n2] = n2 < NL ? fx_of<fx_head(R2)>(raw[n2 < NL ? n2 : 0], et) : mk(0ll, 0ll);
+  const int et = block_in<R2, NL>(v, raw, m);
+  const bool some = m != 0;
   dft_maybe_half<R2, INV, HALF>(v);
   __syncthreads();  // twiddles staged, units cleared
   const int u = fx_unit_of(et, fx_head(R2)) + 2;
@@ -124,7 +147,7 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
     v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<INV>(v[k2], tw[n1 * k2]);
     m = fx_or(fx_or(m, v[k2].x), v[k2].y);
   }
-  column_max<TC, NT>(unit, want_unit<R1>(u, m));
+  column_max<TC, NT>(unit, some ? want_unit<R1>(u, m) : kNoUnit);
   __syncthreads();
   const int U = unit[c];
   to_unit<R2>(v, u, U);
@@ -136,13 +159,14 @@ __global__ void __launch_bounds__(TC * R1) ypass_kernel(const YArgs a) {
 #pragma unroll
     for (int i = 0; i < R1; ++i) w[i] = sm[n1 * S2 + i * TC + c];
     DFT<R1, INV, fxc>::run(w);
-    if (colok) {
+    if (colok)
+      by_unit(plain_unit(U), [&](auto plain) {
 #pragma unroll
-      for (int k1 = 0; k1 < (PAD && INV ? R1 / 2 : R1); ++k1) {
-        const int row = n1 + R2 * k1;
-        if (!INV || (row >= a.ylo && row < a.yhi)) col[(size_t)row * a.sx] = dbl_of(w[k1], U);
-      }
-    }
+        for (int k1 = 0; k1 < (PAD && INV ? R1 / 2 : R1); ++k1) {
+          const int row = n1 + R2 * k1;
+          if (!INV || (row >= a.ylo && row < a.yhi)) col[(size_t)row * a.sx] = dbl_of<plain.value>(w[k1], U);
+        }
+      });
   }
 }
 
@@ -218,7 +242,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
   const size_t cstride = (size_t)a.nzs * zstride;
   double2* col = a.base + (size_t)y * a.sx + kx;
   for (int i = t; i < L; i += NT) tw[i] = a.tw[i];
-  for (int i = t; i < 6 * TC; i += NT) unit[i / TC][i % TC] = INT_MIN;
+  for (int i = t; i < 6 * TC; i += NT) unit[i / TC][i % TC] = kNoUnit;
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) {
     fxc* Fq = F + q * CS;
@@ -232,10 +256,9 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
     }
 #pragma unroll
     for (int n2 = 0; n2 < NL; ++n2) m = top_of(m, raw[n2]);
-    const int et = fx_exp_of(m);
     fxc v[R2];
-#pragma unroll
-    for (int n2 = 0; n2 < R2; ++n2) v[n2] = n2 < NL ? fx_of<fx_head(R2)>(raw[n2 < NL ? n2 : 0], et) : mk(0ll, 0ll);
+    const int et = block_in<R2, NL>(v, raw, m);
+    const bool some = m != 0;
     dft_maybe_half<R2, false, PR>(v);
     if (q == 0) __syncthreads();  // twiddles staged, units cleared
     const int u = fx_unit_of(et, fx_head(R2)) + 2;
@@ -245,7 +268,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<false>(v[k2], tw[n1 * k2]);
       m = fx_or(fx_or(m, v[k2].x), v[k2].y);
     }
-    column_max<TC, NT>(unit[q], want_unit<R1>(u, m));
+    column_max<TC, NT>(unit[q], some ? want_unit<R1>(u, m) : kNoUnit);
     __syncthreads();
     to_unit<R2>(v, u, unit[q][c]);
 #pragma unroll
@@ -374,23 +397,26 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) v[k2] = Fq[n1 * S1 + k2 * TC + c];
     DFT<R2, true, fxc>::run(v);
-    if (colok) {
+    if (colok)
+      by_unit(plain_unit(U), [&](auto plain) {
 #pragma unroll
-      for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) {
-        const int l = n1 + R1 * m2;
-        if (PR != TB || (l >= a.olo && l < a.ohi)) col[q * cstride + l * zstride] = dbl_of(v[m2], U);
-      }
-    }
+        for (int m2 = 0; m2 < (PR ? R2 / 2 : R2); ++m2) {
+          const int l = n1 + R1 * m2;
+          if (PR != TB || (l >= a.olo && l < a.ohi)) col[q * cstride + l * zstride] = dbl_of<plain.value>(v[m2], U);
+        }
+      });
   }
 }
 
 // ---------------------------------------------------------------- x passes
 // As xwide_kernel (passes_wide.cuh), with the transforms in fixed point.  The rows between the
 // transforms are doubles in shared memory.
-// SPLIT: each work item is one component of a tile (the passes that multiply by chi).
+// SPLIT: each work item is one component of a tile (the passes that multiply by chi).  The power-law,
+// assemble and update passes whose C2R is R1i 16 points are held to six CTAs an SM (168 registers): left alone
+// they take 188 to 210 (64 x 64 x 96: update 89 us against 63, power law 117 against 107).
 template <int CIN, int COUT, int R1i, int R2i, int R2o, bool SPLIT>
-__global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const int4* __restrict__ tw_in,
-                                                   const int4* __restrict__ tw_out) {
+__global__ void __launch_bounds__(64, R1i <= 8 && R2i == 16 && CIN > 0 && COUT == 1 ? 6 : 0)
+    xpass_kernel(const XArgs<double> a, const int4* __restrict__ tw_in, const int4* __restrict__ tw_out) {
   typedef WX<CIN, COUT, R1i, R2i, R2o> S;
   constexpr int TP = S::TP, P = S::P, NT = S::NT, XL = S::XL, TT = S::TT, Li = S::Li, Lo = S::Lo, R1o = S::R1o;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -426,7 +452,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
 #pragma unroll 1
       for (int q = q0; q < q1; ++q) {
         fxc v[R2i];
-        int u = INT_MIN, want = INT_MIN;
+        int u = kNoUnit, want = kNoUnit;
         if (r < R1i) {
           const double2* ra = a.spec_in + ((size_t)(q * nz + z) * a.in_rows + ya) * a.in_sx;
           const double2* rb = ra + a.in_sx;
@@ -445,9 +471,8 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
             raw[n2] = raw_of(lo ? make_double2(A.x - B.y, A.y + B.x) : make_double2(A.x + B.y, B.x - A.y));
             m = top_of(m, raw[n2]);
           }
-          const int et = fx_exp_of(m);
-#pragma unroll
-          for (int n2 = 0; n2 < R2i; ++n2) v[n2] = fx_of<fx_head(R2i)>(raw[n2], et);
+          const int et = block_in<R2i, R2i>(v, raw, m);
+          const bool some = m != 0;
           DFT<R2i, true, fxc>::run(v);
           u = fx_unit_of(et, fx_head(R2i)) + 2;
           m = 0;
@@ -456,7 +481,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
             v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<true>(v[k2], twi[k2 * R1i + r]);
             m = fx_or(fx_or(m, v[k2].x), v[k2].y);
           }
-          want = want_unit<R1i>(u, m);
+          if (some) want = want_unit<R1i>(u, m);
         }
 #pragma unroll
         for (int o = 1; o < TP; o <<= 1) want = max(want, __shfl_xor_sync(0xffffffffu, want, o));
@@ -471,8 +496,10 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
 #pragma unroll
           for (int i = 0; i < R1i; ++i) w[i] = Tp[r * (R1i + 1) + i];
           DFT<R1i, true, fxc>::run(w);
+          by_unit(plain_unit(want), [&](auto plain) {
 #pragma unroll
-          for (int k1 = 0; k1 < S::KX; ++k1) RS[(q * P + p) * XL + r + R2i * k1] = dbl_of(w[k1], want);
+            for (int k1 = 0; k1 < S::KX; ++k1) RS[(q * P + p) * XL + r + R2i * k1] = dbl_of<plain.value>(w[k1], want);
+          });
         }
         __syncwarp();
       }
@@ -538,7 +565,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
         constexpr bool HALF = COUT == 2;
         constexpr int NL = HALF ? R2o / 2 : R2o;
         fxc v[R2o];
-        int u = INT_MIN, want = INT_MIN;
+        int u = kNoUnit, want = kNoUnit;
         if (r < R1o) {
           int4 raw[NL];
           int m = 0;
@@ -547,9 +574,8 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
             raw[n2] = ld_raw(RS + (q * P + p) * XL + r + R1o * n2);
             m = top_of(m, raw[n2]);
           }
-          const int et = fx_exp_of(m);
-#pragma unroll
-          for (int n2 = 0; n2 < R2o; ++n2) v[n2] = n2 < NL ? fx_of<fx_head(R2o)>(raw[n2 < NL ? n2 : 0], et) : mk(0ll, 0ll);
+          const int et = block_in<R2o, NL>(v, raw, m);
+          const bool some = m != 0;
           dft_maybe_half<R2o, false, HALF>(v);
           u = fx_unit_of(et, fx_head(R2o)) + 2;
           m = 0;
@@ -558,7 +584,7 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
             v[k2] = k2 == 0 ? fx_quarter(v[0]) : fx_twiddle<false>(v[k2], two[k2 * R1o + r]);
             m = fx_or(fx_or(m, v[k2].x), v[k2].y);
           }
-          want = want_unit<R1o>(u, m);
+          if (some) want = want_unit<R1o>(u, m);
         }
 #pragma unroll
         for (int o = 1; o < TP; o <<= 1) want = max(want, __shfl_xor_sync(0xffffffffu, want, o));
@@ -584,17 +610,19 @@ __global__ void __launch_bounds__(64) xpass_kernel(const XArgs<double> a, const 
         const int src = lane - k2 + (k2 == 0 ? 0 : (k2 < R2o ? R2o - k2 : k2));
         double2* ra = a.spec_out + ((size_t)(q * nz + z) * a.out_rows + ya) * a.out_sx;
         double2* rb = ra + a.out_sx;
+        by_unit(__all_sync(0xffffffffu, plain_unit(want - 1)), [&](auto plain) {  // (the lanes shuffle together)
 #pragma unroll
-        for (int k1 = 0; k1 <= R1o / 2; ++k1) {
-          const fxc sh = shfl_fx(Zr[R1o - 1 - k1], src);
-          const fxc Zk = Zr[k1];
-          const fxc Zm = k2 == 0 ? Zr[(R1o - k1) % R1o] : sh;
-          const int k = k2 + R2o * k1;
-          if (k2 < R2o && pok && k <= Lo / 2) {
-            ra[k] = dbl_of(mk(Zk.x + Zm.x, Zk.y - Zm.y), want - 1);
-            rb[k] = dbl_of(mk(Zk.y + Zm.y, Zm.x - Zk.x), want - 1);
+          for (int k1 = 0; k1 <= R1o / 2; ++k1) {
+            const fxc sh = shfl_fx(Zr[R1o - 1 - k1], src);
+            const fxc Zk = Zr[k1];
+            const fxc Zm = k2 == 0 ? Zr[(R1o - k1) % R1o] : sh;
+            const int k = k2 + R2o * k1;
+            if (k2 < R2o && pok && k <= Lo / 2) {
+              ra[k] = dbl_of<plain.value>(mk(Zk.x + Zm.x, Zk.y - Zm.y), want - 1);
+              rb[k] = dbl_of<plain.value>(mk(Zk.y + Zm.y, Zm.x - Zk.x), want - 1);
+            }
           }
-        }
+        });
         __syncwarp();  // the next component's first stage overwrites Tp
       }
     }

@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
   double2* col = a.base + (size_t)y * a.sx + kx;
   for (int i = t; i < L; i += NT) tw[i] = a.tw[i];
   for (int i = t; i < 6 * TC; i += NT) unit[i / TC][i % TC] = kNoUnit;
+  bool z0 = true, z1 = true;  // whether the x, the y component has anything on the thread's points that k_z multiplies
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) {
     fxc* Fq = F + q * CS;
@@ -281,6 +282,14 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       DFT<R1, false, fxc>::run(w);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) Fq[n1 * S2 + k1 * TC + c] = w[k1];
+      if (!PR) {
+        long long any = 0;
+#pragma unroll
+        for (int k1 = 0; k1 < R1; ++k1)
+          if (k1 % (R1 / 2) != 0 || n1 != 0) any |= w[k1].x | w[k1].y;  // (k_z = 0 on DC and Nyquist)
+        if (q == 0) z0 = any != 0;
+        if (q == 1) z1 = any != 0;
+      }
     }
   }
   // product at kz = k2 + R2 k1 on the thread's own slots: G = i (k x F), |k| < 2^62 in units 2^(ec-62)
@@ -290,7 +299,7 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
     const int k2 = n1;
     fxc* F0 = F + k2 * S2 + c;
     const int u0 = unit[0][c], u1 = unit[1][c], u2 = unit[2][c];
-    const int ux = u1 > u2 ? u1 : u2, uy = u0 > u2 ? u0 : u2, uz = u0 > u1 ? u0 : u1;
+    int ux = u1 > u2 ? u1 : u2, uy = u0 > u2 ? u0 : u2, uz = u0 > u1 ? u0 : u1;
     int ec;
     long long cx = 0, cy = 0, cz = 0;
     const size_t plane = (size_t)(a.ny + 1) * (a.nx + 1), oct = plane * (a.nz + 1);
@@ -306,14 +315,25 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       cy = scaled62(dy, ec - a.e1);
       cz = scaled62(s, ec - a.e2);
     }
+    // A spectrum whose factor vanishes has no part in the unit of the product (the curl on k_x = 0 or k_y = 0, and
+    // off the DC of a component that does not vary along z: a uniform background must not cost the rest its
+    // low bits).  An infinity or a NaN has, as 0 times it is a NaN.
+    const bool tx = PR || cx != 0, ty = PR || cy != 0;
+    if (!PR) {
+      auto take = [](int u, bool on) { return on || u >= kNanUnit / 2 ? u : kNoUnit; };
+      ux = max(take(u1, z1), take(u2, ty));
+      uy = max(take(u2, tx), take(u0, z0));
+      uz = max(take(u0, ty), take(u1, tx));
+    }
     ug[0] = ux + ec + 2;
     ug[1] = uy + ec + 2;
     ug[2] = uz + ec + 2;
     if (n1 < R2) {
       // right shifts that bring the two spectra of an output to their common unit, taken on the
       // factors, which have bits to spare
-      const int s1x = min(ux - u1, 63), s2x = min(ux - u2, 63), s0y = min(uy - u0, 63), s2y = min(uy - u2, 63),
-                s0z = min(uz - u0, 63), s1z = min(uz - u1, 63);
+      auto shift = [](int U, int u, bool on) { return PR || on ? min(U - u, 63) : 63; };
+      const int s1x = shift(ux, u1, z1), s2x = shift(ux, u2, ty), s0y = shift(uy, u0, z0), s2y = shift(uy, u2, tx),
+                s0z = shift(uz, u0, ty), s1z = shift(uz, u1, tx);
 #pragma unroll 2
       for (int k1 = 0; k1 < R1; ++k1) {
         const int kz = k2 + R2 * k1;

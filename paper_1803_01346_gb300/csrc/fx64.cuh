@@ -13,9 +13,10 @@
 //   Stage B: the blocks that meet in it (the threads of one pencil) are brought to a common unit,
 //     the finest in which the largest value still stays below 2^head(R).
 // Rounding therefore happens at 2^-57 or so of the largest value of a block instead of at 2^-53 of
-// each value, and additions are exact: against exact arithmetic the transform of 16 to 256 points
-// comes out 2 to 4 times nearer than the FP64 one (what is left is the rounding of the results to
-// doubles).  A block that holds an infinity or a NaN gives NaN (unit kNanUnit).
+// each value, and additions are exact: against long double the transform of 16 to 256 points comes
+// out 1.8 to 3.6 times nearer (relative 2-norm) than the same two stages in FP64: 1.9 to 3.3 for white and
+// zero-padded pencils, 1.8 to 2.8 for spikes and for spectra that fall off (what is left is the
+// rounding of the results to doubles).  A block that holds an infinity or a NaN gives NaN (unit kNanUnit).
 // Subnormal doubles are read and written (a unit below that of the smallest normal is as good as any).
 //
 // Unit exponents are kept in the bias of FP64: value = v 2^(u - 1075).

@@ -264,3 +264,10 @@ def test_pencils_of_any_exponent_keep_their_accuracy(tmp_path):
     rounding of two stages at 2^-57 of the largest value and of the result to a double stay below 2^-53."""
     for L, inv, _, scale, fx, _ in pencils(tmp_path, 1, (0, 900, -900, -960, -980, -1000, -1010)):
         assert fx < 2.0 ** -53, (L, inv, scale, fx)
+
+
+def test_pencils_are_nearer_to_exact_than_in_fp64(tmp_path):
+    """The rounding of a pencil's largest value at 2^-57 in two stages adds less than the rounding of each
+    value at 2^-53 in every butterfly does, whatever the spectrum."""
+    for L, inv, kind, _, fx, fp64 in pencils(tmp_path, 6, (0,)):
+        assert fx < fp64, (L, inv, kind, fx, fp64)

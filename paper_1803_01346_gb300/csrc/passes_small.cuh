@@ -7,7 +7,8 @@
 // of a warp, one to a lane (two for 64 points), and a butterfly is a shuffle and one instruction
 // for each part: 16 points are about 16 FP64 instructions deep, 32 points 18, against 160 and 116
 // for a thread that transforms 16 or 8 points in its registers.  Measured on 16^3: one curl 55.3 ->
-// 22.3 us, an adaptive run 42.3 -> 23.1 ms.  The y and z passes of 64 points (32^3 and its like on the
+// 22.3 us, an adaptive run 42.3 -> 23.1 ms (12.1 us and 12.7 ms since the passes follow each other as
+// dependent launches and the Eq. 5 loop is a graph).  The y and z passes of 64 points (32^3 and its like on the
 // padded grid) have enough warps, so what counts is the number of instructions, about 17 a
 // point with 8 points to a thread against 24 in lanes, and they keep that form.
 // The operations are those of the register transforms (fft_core.cuh: 16 = 4 x 4, 32 = 4 x 8,
@@ -330,7 +331,7 @@ struct ZArgs {
   int nx, ny, nz;
   const Ctrl* ctrl;
   int check_done;
-  int ilo, ihi, olo, ohi;  // planes outside [ilo, ihi) read as zero, planes outside [olo, ohi) are not written
+  int ilo, ihi, olo, ohi;  // planes outside [ilo, ihi) read as zero, planes outside [olo, ohi) need not be written
 };
 // 16 and 32 points: one CTA of three warps, a component to a warp, for two or one columns (kx, y);
 // the three spectra meet in shared memory, where each thread takes the product of its own component.

@@ -9,7 +9,7 @@
 
 namespace scfft {
 
-constexpr int kThreads = 256;  // every FFT pass kernel runs 256-thread CTAs
+constexpr int kThreads = 256;  // CTAs of the node-wise kernels (finalize, conversions, kernel spectrum)
 
 // Allow a kernel the largest dynamic shared memory a CTA may use, once per
 // kernel (thread-safe static initialisation).  Raising the cap once, instead of
@@ -54,10 +54,17 @@ struct Geo {
 };
 
 // FP64: whether the grid's passes run in 64-bit fixed point (passes_fx.cuh) or, with every axis at
-// most 32, in native FP64 (passes_small.cuh): there both are bound by latency and about as fast
-// (one 16^3 curl 55 us native, 48 us fixed; the 64 x 64 x 96 right-hand side 9.6 ms native with the
-// same structure, 3.3 ms fixed), and the native passes keep the rounding that the small grids'
-// step sequences were recorded with.
+// most 32, in native FP64 across the lanes of a warp (passes_small.cuh).  Small grids are bound by latency,
+// and the lanes' chains are the shorter ones; with more than 32 points an axis the FP64 pipe binds (the
+// native passes end there: 64 x 64 x 96, one right-hand side 9.6 ms native with the fixed-point passes'
+// structure, 2.8 fixed).  Measured, us a call, native | fixed point:
+//             16^3       32x16x16   32x32x16   16x32x32   32^3
+//   curl      12 | 26    13 | 31    14 | 33    16 | 32    20 | 37
+//   Phi       15 | 31    22 | 35    35 | 38    38 | 40    62 | 45
+//   rhs      167 | 289  191 | 331  291 | 403  253 | 330  415 | 451
+// The line lies at 32 for whole right-hand sides: only Phi alone and the stencil curl's right-hand side
+// (573 | 462) would gain at 32^3.  The native passes also keep the last bits that a small grid's step
+// sequence depends on.
 inline bool fixed_point_grid(const Geo& g) { return g.nx > 32 || g.ny > 32 || g.nz > 32; }
 
 // TMA descriptors of the FP32 padded y passes: the padded half spectrum Pd as read by the
@@ -91,11 +98,13 @@ struct Work {
   float4* kap4 = nullptr; // FP32 only: the same octant interleaved, [nz+1][ny+1][nx+1] x {a=0,1,2, 0}
   T* kt[3] = {nullptr, nullptr, nullptr};  // derivative wavenumbers (0 on Nyquist): nx/2+1, ny, nz
   T* st[3] = {nullptr, nullptr, nullptr};  // Gaussian smoothing factor per axis: nx/2+1, ny, nz
-  V* twu[3] = {nullptr, nullptr, nullptr}; // twiddles W_L^m, L = nx, ny, nz
-  V* twp[3] = {nullptr, nullptr, nullptr}; // twiddles, L = 2nx, 2ny, 2nz
+  // twiddles W_L^m, L = nx, ny, nz and L = 2nx, 2ny, 2nz (null in FP64 on grids of the fixed-point passes, which
+  // take fxu and fxp)
+  V* twu[3] = {nullptr, nullptr, nullptr};
+  V* twp[3] = {nullptr, nullptr, nullptr};
   YMaps* ym = nullptr;   // FP32 only: TMA descriptors of the y passes (nullptr: plain-load y passes)
-  // FP64 only (fixed-point passes, fx64.cuh; kap as integers only on grids that take them): twiddles 2^62 (cos, sin) as 32-bit halves for L = n
-  // and L = 2n per axis; S and S k along z as integers with their exponents; exponent of a kernel
+  // FP64 only, on grids of the fixed-point passes (fx64.cuh): twiddles 2^62 (cos, sin) as 32-bit halves for
+  // L = n and L = 2n per axis; S and S k along z as integers with their exponents; exponent of a kernel
   // spectrum's column (ky, kx), whose values kap holds as integers K 2^(62 - ek)
   int4* fxu[3] = {nullptr, nullptr, nullptr};
   int4* fxp[3] = {nullptr, nullptr, nullptr};
@@ -176,8 +185,8 @@ struct Launch {
 // kernel that has ended implies that all before it have.)  Measured: 16^3 FP64 curl 22.3 -> 12.1 us, Phi
 // 48 x 32 x 128 FP32 57.1 -> 45.8, reverse mode 48^3 FP64 1251 -> 1109 us.  No pass signals
 // before it ends (griddepcontrol.launch_dependents): the next one's CTAs then fill
-// the SMs that drain first and sit there unevenly (rhs 64 x 64 x 96 FP64 3.55 ms against 3.15 with
-// the signal left to the end, 3.28 without any of this).
+// the SMs that drain first and sit there unevenly (rhs 64 x 64 x 96 FP64, when it took 3.28 ms without
+// any of this: 3.55 with the early signal, 3.15 with the signal left to the end).
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

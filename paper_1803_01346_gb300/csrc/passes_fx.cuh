@@ -315,15 +315,20 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
       cy = scaled62(dy, ec - a.e1);
       cz = scaled62(s, ec - a.e2);
     }
-    // A spectrum whose factor vanishes has no part in the unit of the product (the curl on k_x = 0 or k_y = 0, and
-    // off the DC of a component that does not vary along z: a uniform background must not cost the rest its
-    // low bits).  An infinity or a NaN has, as 0 times it is a NaN.
-    const bool tx = PR || cx != 0, ty = PR || cy != 0;
+    // A spectrum whose factor vanishes does not set the unit of the product when the other one would lose bits by
+    // it (the curl on k_x = 0 or k_y = 0, and off the DC of a component that does not vary along z: a uniform
+    // background must not cost the rest its low bits; within 2^4 of each other nothing is lost, the factors having
+    // 62).  An infinity or a NaN does, as 0 times it is a NaN.
     if (!PR) {
-      auto take = [](int u, bool on) { return on || u >= kNanUnit / 2 ? u : kNoUnit; };
-      ux = max(take(u1, z1), take(u2, ty));
-      uy = max(take(u2, tx), take(u0, z0));
-      uz = max(take(u0, ty), take(u1, tx));
+      const bool tx = cx != 0, ty = cy != 0;
+      auto unit_of = [](int ua, bool a_on, int ub, bool b_on) {
+        if (!a_on && b_on && ua > ub + 4 && ua < kNanUnit / 2) return ub;
+        if (a_on && !b_on && ub > ua + 4 && ub < kNanUnit / 2) return ua;
+        return max(ua, ub);
+      };
+      ux = unit_of(u1, z1, u2, ty);
+      uy = unit_of(u2, tx, u0, z0);
+      uz = unit_of(u0, ty, u1, tx);
     }
     ug[0] = ux + ec + 2;
     ug[1] = uy + ec + 2;
@@ -331,9 +336,9 @@ __global__ void __launch_bounds__(TC * R1) zpass_kernel(const ZArgs a) {
     if (n1 < R2) {
       // right shifts that bring the two spectra of an output to their common unit, taken on the
       // factors, which have bits to spare
-      auto shift = [](int U, int u, bool on) { return PR || on ? min(U - u, 63) : 63; };
-      const int s1x = shift(ux, u1, z1), s2x = shift(ux, u2, ty), s0y = shift(uy, u0, z0), s2y = shift(uy, u2, tx),
-                s0z = shift(uz, u0, ty), s1z = shift(uz, u1, tx);
+      auto shift = [](int U, int u) { return PR || U >= u ? min(U - u, 63) : 63; };
+      const int s1x = shift(ux, u1), s2x = shift(ux, u2), s0y = shift(uy, u0), s2y = shift(uy, u2), s0z = shift(uz, u0),
+                s1z = shift(uz, u1);
 #pragma unroll 2
       for (int k1 = 0; k1 < R1; ++k1) {
         const int kz = k2 + R2 * k1;

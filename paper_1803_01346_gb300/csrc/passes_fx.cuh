@@ -3,15 +3,15 @@
 // node-wise steps in FP64.
 //
 // What bounds them is latency and issue on the integer pipes (additions 2, twiddles about 20
-// instructions a point): the padded z pass runs 10 warps an SM, by shared memory and registers, at 41%
-// issue, the y passes 16 to 20 warps at 55 to 60%; not the FP64 pipe, which kept the FP64 passes
-// before these 76% busy.  Measured on 64 x 64 x 96 with a shield's box, us a launch, FP64 |
-// double-float passes before | these: padded z 589 | 306 | 141, Eq. 5 update 177 | 122 | 65, padded y
-// inverse 127 | 71 | 33, curl z 79 | 51 | 33; one right-hand side 10.4 | 6.2 | 2.9 ms.  A length L = R1 R2
+// instructions a point): the padded z pass of 192 points runs 8 warps an SM (211 registers) at 46% issue, the
+// y passes 19 warps at 60%; not the FP64 pipe, which kept the FP64 passes before these 76% busy.
+// Measured on 64 x 64 x 96 with a shield's box, us a launch, FP64 |
+// double-float passes before | these: padded z 589 | 306 | 136, Eq. 5 update 177 | 122 | 63, padded y
+// inverse 127 | 71 | 32, curl z 79 | 51 | 32; one right-hand side 10.4 | 6.2 | 2.8 ms.  A length L = R1 R2
 // transform is two register stages with one shared-memory transpose; every length is compiled on its
 // own; the component loops stay rolled, so that a kernel's four unrolled DFT bodies stay within the
-// instruction cache.  (Reading a component's input during the transform before it, in the z pass: 141 us
-// either way.)
+// instruction cache.  (Reading a component's input during the transform before it, in the z pass: no gain.
+// The z pass of 192 points held to five CTAs an SM, 200 registers: Phi 96^3's 314 us against 292.)
 #pragma once
 #include <limits.h>
 
@@ -204,7 +204,7 @@ __device__ __forceinline__ long long scaled62(double c, int e) {
 // unpadded grid; KIND 1: the Biot-Savart kernel on the padded grid (half of the input planes are
 // zero and half of the output planes are kept).  Omega's box: KIND 1 reads and KIND 0 writes its
 // planes only; TB, the transposed iteration's form, the other way round (run-time ranges on both
-// sides of both cost Phi 96^3 557 us against 552).  A 1-D grid: TC consecutive kx of one row per
+// sides of both cost Phi 96^3 1%).  A 1-D grid: TC consecutive kx of one row per
 // CTA; the columns left over when HX is not a multiple of TC are packed TC (row, kx) pairs to a
 // CTA and run first.
 template <int R1, int R2, int TC, int KIND, bool TB>
